@@ -567,7 +567,12 @@ ps_status ps_init(const ps_params* p, void* cuda_stream, void* workspace_dev, si
     kp.invn3 = 1.0 / ((double)n * n * nz);
     kp.dx = p->L / n;
     kp.half_L3 = 0.5 * p->L * p->L * Lz;
-    for (int i = 0; i < 3; ++i) kp.x0[i] = p->x0[i];
+    for (int i = 0; i < 3; ++i) {
+        kp.x0[i] = p->x0[i];
+        const double j = rint(p->x0[i] / kp.dx), jmax = i == 2 ? nz : n;
+        kp.jc[i] = j > 0.0 ? (j < jmax ? (int)j : (int)jmax) : 0;
+        kp.jo[i] = kp.jc[i] * kp.dx - p->x0[i];
+    }
     kp.mean_free = p->mean_mode == PS_MEAN_FREE;
 
     unsigned char* w = (unsigned char*)workspace_dev;

@@ -95,6 +95,8 @@ struct KP {
     double ksz;       // 2 pi / Lz (Lz = L nz / n: the same spacing on every axis)
     double dt, inv_eta, invn3, dx, half_L3;
     double x0[3];
+    int jc[3];        // grid point next to x0 (clamped to the grid): moments are summed about it in
+    double jo[3];     // whole cells, jo = jc dx - x0 moves them to x0
     int mean_free;
     int xs0, xsn;     // x planes [xs0, xs0 + xsn) handled by the y and z passes
     int ky0, kyn;     // kept ky rows [ky0, ky0 + kyn) handled by the TMA x passes (slab decomposition)
@@ -117,6 +119,50 @@ struct Acc {
     }
     __device__ __forceinline__ double val() const { return s + c; }
 };
+
+// Penalization sums of the z pass: q = chi (u - u_s) of a point and a thread's
+// running sums of q and of whole-cell offsets times q. FP64 fields: doubles.
+// FP32 fields: unevaluated FP32 pairs (h + l, about 48 bits: exact difference
+// and product by two-sum and fused multiply-add, the rounding of l is the
+// error), summed over the few points a thread has in a batch and over its
+// warp, then added to the compensated doubles. An FP64 instruction takes 64
+// cycles of a quarter SM, an FP32 one a cycle: with the sums in doubles from
+// the point on, 31 FP64 instructions per masked point and 66 per warp made up
+// most of the pass where the mask fills many lines (GB300: static plate at
+// 128^3 83 -> 42 us per pass, wing at 48^3 17 -> 11 us, at 256^3 173 -> 164).
+struct Pair32 {
+    float h, l;
+};
+__device__ __forceinline__ Pair32 pair_sum(float a, float b) {   // a + b exactly
+    const float s = __fadd_rn(a, b), t = __fadd_rn(s, -a);
+    return {s, __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -t)), __fadd_rn(b, -t))};
+}
+__device__ __forceinline__ Pair32 pair_mul(float j, Pair32 q) {
+    const float h = __fmul_rn(j, q.h);
+    return {h, __fmaf_rn(j, q.l, __fmaf_rn(j, q.h, -h))};
+}
+__device__ __forceinline__ void sum_add(Pair32& a, Pair32 q) {
+    const Pair32 s = pair_sum(a.h, q.h);
+    a.h = s.h;
+    a.l = __fadd_rn(a.l, __fadd_rn(s.l, q.l));
+}
+__device__ __forceinline__ void sum_add(double& a, double q) { a += q; }
+__device__ __forceinline__ void sum_fma(Pair32& a, float j, Pair32 q) { sum_add(a, pair_mul(j, q)); }
+__device__ __forceinline__ void sum_fma(double& a, double j, double q) { a = fma(j, q, a); }
+__device__ __forceinline__ Pair32 pen_term(float c, float u, float s) { return pair_mul(c, pair_sum(u, -s)); }
+__device__ __forceinline__ double pen_term(double c, double u, double s) { return c * (u - s); }
+__device__ __forceinline__ double sum_val(Pair32 a) { return (double)a.h + (double)a.l; }
+__device__ __forceinline__ double sum_val(double a) { return a; }
+__device__ __forceinline__ Pair32 sum_down(unsigned m, Pair32 a, int o) {
+    return {__shfl_down_sync(m, a.h, o), __shfl_down_sync(m, a.l, o)};
+}
+__device__ __forceinline__ double sum_down(unsigned m, double a, int o) { return __shfl_down_sync(m, a, o); }
+__device__ __forceinline__ Pair32 sum_from0(unsigned m, Pair32 a) {
+    return {__shfl_sync(m, a.h, 0), __shfl_sync(m, a.l, 0)};
+}
+__device__ __forceinline__ double sum_from0(unsigned m, double a) { return __shfl_sync(m, a, 0); }
+template <typename T> struct sum_of { using type = Pair32; };
+template <> struct sum_of<double> { using type = double; };
 
 // Block-wide sum of `nv` doubles per thread into out[0..nv) (thread 0 writes).
 template <int NV>
@@ -698,9 +744,10 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
         __syncthreads();
         // one buffer: every read of it is done, the next batch may land
         if (!Z3 && NB == 1 && threadIdx.x == 0 && more) issue(b + gridDim.x, 0);
-        double fm[6] = {0, 0, 0, 0, 0, 0};
+        using Sum = typename sum_of<T>::type;
+        Sum fm[6] = {};   // q and (offset from jc in cells) x q
         bool touched = false;
-        // n = u x w - (chi/eta)(u - us) of line l at z; forces in double
+        // n = u x w - (chi/eta)(u - us) of line l at z and the force sums
         auto nonlinear = [&](int l, int z, int a, T& nx, T& ny, T& nz) {
             const long lid = (long)b * LZ + l;
             const C2 z0 = tile(l, 0)[a], z1 = tile(l, 1)[a], z2 = tile(l, 2)[a];
@@ -719,17 +766,19 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
                     nx -= ce * (ux - sx);
                     ny -= ce * (uy - sy);
                     nz -= ce * (uz - sz);
-                    const double cd = (double)c;
-                    const double px = cd * ((double)ux - (double)sx);
-                    const double py = cd * ((double)uy - (double)sy);
-                    const double pz = cd * ((double)uz - (double)sz);
-                    const double rx = x * kp.dx - kp.x0[0], ry = y * kp.dx - kp.x0[1], rz = z * kp.dx - kp.x0[2];
-                    fm[0] += px;
-                    fm[1] += py;
-                    fm[2] += pz;
-                    fm[3] += ry * pz - rz * py;
-                    fm[4] += rz * px - rx * pz;
-                    fm[5] += rx * py - ry * px;
+                    if constexpr (!PM) {
+                        const Sum qx = pen_term(c, ux, sx), qy = pen_term(c, uy, sy), qz = pen_term(c, uz, sz);
+                        const T jx = (T)(x - kp.jc[0]), jy = (T)(y - kp.jc[1]), jz = (T)(z - kp.jc[2]);
+                        sum_add(fm[0], qx);
+                        sum_add(fm[1], qy);
+                        sum_add(fm[2], qz);
+                        sum_fma(fm[3], jy, qz);
+                        sum_fma(fm[3], -jz, qy);
+                        sum_fma(fm[4], jz, qx);
+                        sum_fma(fm[4], -jx, qz);
+                        sum_fma(fm[5], jx, qy);
+                        sum_fma(fm[5], -jy, qx);
+                    }
                     touched = true;
                 }
             }
@@ -759,19 +808,33 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
             tile(l + 1, 0)[a] = cmk<C2>(nx1, ny1);
             tile(l, 1)[a] = cmk<C2>(nz0, nz1);
         }
-        // this batch's force sums: warp tree, then compensated into the warp slot
-        if (__any_sync(0xffffffffu, touched)) {
-            for (int i = 0; i < 6; ++i)
-                for (int o = 16; o > 0; o >>= 1) fm[i] += __shfl_down_sync(0xffffffffu, fm[i], o);
-            if ((threadIdx.x & 31) == 0) {
-                double* w = wacc[threadIdx.x >> 5];
-                for (int i = 0; i < 6; ++i) {
-                    Acc a = {w[2 * i], w[2 * i + 1]};
-                    a.add(fm[i]);
-                    w[2 * i] = a.s;
-                    w[2 * i + 1] = a.c;
+        // this batch's force sums: warp tree over the lanes that exist, then
+        // lane i < 6 adds sum i, compensated, to the warp's slot
+        if (!PM && __any_sync(warp_lanes(), touched)) {
+            constexpr int TAIL = 3 * LZ * G % 32;   // lanes of a last, partial warp
+            static_assert(TAIL == 0 || TAIL >= 3, "two sums per lane at most");
+            const unsigned m = warp_lanes();
+            const int lane = threadIdx.x & 31, nl = __popc(m);
+            Sum mine[2] = {};   // the second of a lane only in a warp of fewer than six
+#pragma unroll
+            for (int i = 0; i < 6; ++i) {
+                for (int o = 16; o > 0; o >>= 1) {
+                    const Sum v = sum_down(m, fm[i], o);
+                    if (lane + o < nl) sum_add(fm[i], v);
                 }
+                const Sum v = sum_from0(m, fm[i]);
+                if (lane == i) mine[0] = v;
+                if (TAIL > 0 && TAIL < 6 && lane + nl == i) mine[1] = v;
             }
+            double* const ws = wacc[threadIdx.x >> 5];
+            auto flush = [&](int i, Sum v) {
+                Acc a = {ws[2 * i], ws[2 * i + 1]};
+                a.add(sum_val(v));
+                ws[2 * i] = a.s;
+                ws[2 * i + 1] = a.c;
+            };
+            if (lane < 6) flush(lane, mine[0]);
+            if (TAIL > 0 && TAIL < 6 && lane + nl < 6) flush(lane + nl, mine[1]);
         }
         __syncthreads();
         {
@@ -866,7 +929,16 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
             a.add(wacc[w][2 * threadIdx.x]);
             a.add(wacc[w][2 * threadIdx.x + 1]);
         }
-        partial[(size_t)(kp.part_off + blockIdx.x) * 6 + threadIdx.x] = a.val();
+        // sums about the grid point jc, in cells -> moments about x0
+        __shared__ double fin[6];
+        fin[threadIdx.x] = a.val();
+        __syncwarp(0x3fu);
+        double v = fin[threadIdx.x];
+        if (threadIdx.x >= 3) {
+            const int c0 = (threadIdx.x - 2) % 3, c1 = (threadIdx.x - 1) % 3;
+            v = kp.dx * v + (kp.jo[c0] * fin[c1] - kp.jo[c1] * fin[c0]);
+        }
+        partial[(size_t)(kp.part_off + blockIdx.x) * 6 + threadIdx.x] = v;
     }
 }
 
