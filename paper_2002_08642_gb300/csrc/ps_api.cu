@@ -434,20 +434,32 @@ cudaError_t ps::rasterise(const MaskArgs& a, void* chi, void* us, uint8_t* flag,
         if ((e = cudaMemsetAsync(chi, 0, n3 * sizeof(T), s)) != cudaSuccess) return e;
         if ((e = cudaMemsetAsync(us, 0, 3 * n3 * sizeof(T), s)) != cudaSuccess) return e;
     }
-    // the previous call's points, the line flags, the other list's count
-    // and the node positions
+    // the previous call's points, the line flags, the other list's count,
+    // the node positions and the triangles' boxes
     const int np = par ^ 1;
-    const int cb = (a.n_nodes + 255) / 256 > 8 * kRasterSM ? (a.n_nodes + 255) / 256 : 8 * kRasterSM;
-    k_mask_clear<T><<<cb, 256, 0, s>>>(m, a, par, (T*)chi, (T*)us, flag, n3, n * n);
+    const int most = std::max(std::max(a.n_nodes, 4 * a.n_tri), 256 * 4 * kRasterSM);
+    const int cb = (most + 255) / 256;
     if (a.profile == PS_MASK_TANH) {
+        k_mask_prepare<T, false><<<cb, 256, 0, s>>>(m, a, par, (T*)chi, (T*)us, flag, n3, n * n, 0.0);
         k_mask_dense<T><<<16 * kRasterSM, 128, 0, s>>>(m, a, (T*)chi, (T*)us, flag);
         *par_out = np;  // both lists empty: the next call must clear densely
         return cudaGetLastError();
     }
-    k_mask_tris<T><<<a.n_tri > 0 ? (a.n_tri + 127) / 128 : 1, 128, 0, s>>>(m, a, a.tw + a.h);
-    k_mask_prefix<<<1, 1024, 0, s>>>(m, a);
-    k_mask_scatter1<T><<<16 * kRasterSM, 256, 0, s>>>(m, a, np);
-    if constexpr (sizeof(T) == 8) k_mask_scatter2<T><<<16 * kRasterSM, 256, 0, s>>>(m, a);
+    k_mask_prepare<T, true><<<cb, 256, 0, s>>>(m, a, par, (T*)chi, (T*)us, flag, n3, n * n, a.tw + a.h);
+    // FP32: about 32 warps per SM over the triangles; FP64: eight, a warp's
+    // last, partly filled round of FP64 tests costs as much as a full one;
+    // at least one per triangle (a wing of thousands of small triangles; a
+    // plate of two large ones is split finely)
+    const int per_sm = sizeof(T) == 4 ? 32 : 8;
+    const int wpt = a.n_tri < per_sm * kRasterSM ? per_sm * kRasterSM / a.n_tri : 1;
+    const int pb = (int)(((long)a.n_tri * wpt * 32 + kPairThreads - 1) / kPairThreads);
+    if constexpr (sizeof(T) == 4) {
+        k_mask_pairs<T, kPairOne><<<pb, kPairThreads, 0, s>>>(m, a, np, wpt);
+    } else {
+        k_mask_pairs<T, kPairBound><<<pb, kPairThreads, 0, s>>>(m, a, np, wpt);
+        k_mask_pairs<T, kPairLeast><<<pb, kPairThreads, 0, s>>>(m, a, np, wpt);
+        k_mask_pairs<T, kPairTies><<<pb, kPairThreads, 0, s>>>(m, a, np, wpt);
+    }
     k_mask_eval<T><<<8 * kRasterSM, 256, 0, s>>>(m, a, np, (T*)chi, (T*)us, flag);
     *par_out = np;
     return cudaGetLastError();
@@ -732,6 +744,7 @@ ps_status ps_set_mask_from_nodes(ps_ctx* c, const double* xw, const double* vw, 
     a.x_lo = c->slab ? c->slab_x0 : 0;
     a.x_hi = c->slab ? c->slab_x1 : c->p.n;
     a.dx = c->kp.dx;
+    a.inv_dx = 1.0 / c->kp.dx;
     a.tw = c->p.tw;
     a.h = c->p.h;
     a.profile = c->p.mask_profile;

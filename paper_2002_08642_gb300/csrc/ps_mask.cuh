@@ -9,26 +9,39 @@
 //     barycentric coordinates of the closest point on the closest triangle
 //     (Eq. relative_velocities).
 //
-// Banded (cosine) profile, per call:
-//   clear     zero chi/u_s and reset the per-point keys of the points the
+// Banded (cosine) profile, three kernels per call (five in FP64):
+//   prepare   zero chi/u_s and reset the per-point keys of the points the
 //             previous call touched (list kept in the workspace), clear the
-//             line flags, and the global node positions X_O + R x^(w)
-//             (double);
-//   tris      per triangle (one thread each): grid-index bounding box and
-//             the geometry the pair tests need, in the context precision:
-//             vertex a as grid cell + offset, edges b - a and c - a;
-//   prefix    exclusive prefix sum of the box point counts (one block);
-//   scatter1  for every (triangle, box point) pair with distance < reach:
-//             atomicMin of a 64-bit key (non-negative IEEE values order like
-//             their bit patterns); the first writer appends the point to the
-//             touched list. FP32: the key is the distance bits above the
-//             triangle index, so its minimum also names the winner (exact
-//             ties -> smallest index). FP64: the distance bits alone, and
-//   scatter2  (FP64 only) pairs within a few ulps of the minimum: atomicMin
-//             of the triangle index (near-ties -> smallest index);
+//             line flags; the global node positions X_O + R x^(w) (double);
+//             per triangle the grid-index bounding box and the geometry the
+//             pair tests need, in the context precision;
+//   pairs     a warp per triangle (several where there are few) walks the
+//             points of its box. FP32: for every pair with distance < reach
+//             an atomicMin of a 64-bit key, the squared distance's bits
+//             (non-negative IEEE values order like their bit patterns) above
+//             the triangle index, so that the minimum also names the winner
+//             (exact ties -> smallest index); the first writer appends the
+//             point to the touched list. FP64, three walks:
+//               bound   an upper bound of each point's least squared
+//                       distance, and the touched list, in FP32;
+//               least   its exact value (atomicMin of the bits);
+//               ties    pairs within a few ulps of it: atomicMin of the
+//                       triangle index (near-ties -> smallest index);
 //   evaluate  per touched point: distance and barycentrics recomputed in
 //             double on the winning triangle, chi, u_s, line flags.
 // The distance used to pick the winner is computed in the context precision.
+//
+// What bounds it: launches and FP64 issue (a warp's FP64 instruction takes 64
+// cycles of a quarter SM whatever its lanes do). So the triangles' boxes go
+// with the clearing instead of into a kernel of their own, one axis per lane;
+// a warp owns a triangle, so that no prefix sum over the boxes and no search
+// in it is needed; distances are compared squared (no root), the dot products
+// of the edges are made once per triangle, divisions by constants are
+// products; and the FP64 pair tests run only for the pairs that a FP32 lower
+// bound of the distance leaves, 32 at a time.
+// GB300, each kernel alone on the device, against clear + boxes + prefix sum +
+// pair pass(es) + evaluate: 121 nodes at 48^3 FP32 48 -> 28 us (6 + 5 + 17),
+// 600 nodes at 128^3 FP64 229 -> 107 us (8 + 24 + 29 + 29 + 17).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -40,7 +53,7 @@ namespace ps {
 struct MaskArgs {
     int n, nz;   // grid n x n x nz, spacing dx on every axis
     int x_lo, x_hi;   // x-planes [x_lo, x_hi) rasterised (a slab of the sharded step; 0, n otherwise)
-    double dx, tw, h;
+    double dx, inv_dx, tw, h;
     int profile;
     const double* xw;
     const double* vw;
@@ -53,15 +66,22 @@ struct MaskArgs {
 static constexpr int kMaskMaxTri = 1 << 17;
 static constexpr int kMaskMaxNodes = 1 << 17;
 
-// Per-triangle geometry of the pair tests: vertex a = ca dx + f per axis (ca
-// its grid cell index, f in [0, dx) the rest), edges b - a and c - a; the
-// lengths rounded once from double to T. A grid point minus a is then
-// (i - ca) dx - f, with no double arithmetic per pair.
+// Per-triangle geometry of the pair tests: bounding box dilated by the reach
+// (first grid index and extent per axis); vertex a = ca dx + f per axis (ca
+// its grid cell index, f the rest, about [0, dx)), edges b - a and c - a and
+// their dot products; the lengths rounded once from double to T. A grid point
+// minus a is then (i - ca) dx - f, with no double arithmetic per pair.
+// m, r: a sphere around the triangle (centre relative to a); nrm: the unit
+// normal (0 for a degenerate triangle).
 template <typename T> struct TriGeo {
-    int ca[4];
+    int i0[3], e[3], ca[3];
+    float r;
     T f[3], b[3], c[3];
+    T bb, bc, cc;
+    float m[3], nrm[3];
 };
-static constexpr size_t kTriGeoBytes = 128;   // >= sizeof(TriGeo<double>)
+static constexpr size_t kTriGeoBytes = 160;   // >= sizeof(TriGeo<double>)
+static_assert(sizeof(TriGeo<double>) <= kTriGeoBytes, "triangle geometry slot");
 
 // Workspace: keys (8 B/pt), winner ids (4 B/pt), two touched lists (4 B/pt
 // each), counters, node and triangle scratch.
@@ -69,17 +89,15 @@ inline size_t mask_workspace_bytes(int n, int nz) {
     const size_t n3 = (size_t)n * n * nz;
     auto a = [](size_t x) { return (x + 255) & ~(size_t)255; };
     return a(n3 * 8) + a(n3 * 4) + 2 * a(n3 * 4) + a(64) + a((size_t)kMaskMaxNodes * 3 * 8) +
-           a((size_t)kMaskMaxTri * 8 * 4) + a(((size_t)kMaskMaxTri + 1) * 8) + a((size_t)kMaskMaxTri * kTriGeoBytes);
+           a((size_t)kMaskMaxTri * kTriGeoBytes);
 }
 
 struct MaskWs {
     unsigned long long* key;
     int32_t* win;
     uint32_t* list[2];
-    unsigned long long* cnt;  // [0],[1]: list lengths, [2]: total pairs, [4]: bad-index flag
+    unsigned long long* cnt;  // [0],[1]: list lengths, [4]: bad-index flag
     double* xg;
-    int32_t* box;              // per triangle: i0,j0,k0,ei,ej,ek, point count (+1 pad)
-    unsigned long long* pre;   // exclusive prefix of box sizes (n_tri + 1)
     unsigned char* geo;        // per triangle: TriGeo<T> in kTriGeoBytes
 };
 
@@ -94,8 +112,6 @@ inline MaskWs mask_ws_split(unsigned char* w, int n, int nz) {
     m.list[1] = (uint32_t*)(w + o); o += a(n3 * 4);
     m.cnt = (unsigned long long*)(w + o); o += a(64);
     m.xg = (double*)(w + o); o += a((size_t)kMaskMaxNodes * 3 * 8);
-    m.box = (int32_t*)(w + o); o += a((size_t)kMaskMaxTri * 8 * 4);
-    m.pre = (unsigned long long*)(w + o); o += a(((size_t)kMaskMaxTri + 1) * 8);
     m.geo = w + o;
     return m;
 }
@@ -148,22 +164,127 @@ __device__ __forceinline__ R closest_tri(const R p[3], const R a[3], const R b[3
     return d2s;
 }
 
-template <typename T> struct KeyBits;
-template <> struct KeyBits<float> {
-    static __device__ __forceinline__ unsigned long long of(float d) { return (unsigned long long)__float_as_uint(d); }
-    static __device__ __forceinline__ float val(unsigned long long k) { return __uint_as_float((unsigned)k); }
-};
-template <> struct KeyBits<double> {
-    static __device__ __forceinline__ unsigned long long of(double d) { return (unsigned long long)__double_as_longlong(d); }
-    static __device__ __forceinline__ double val(unsigned long long k) { return __longlong_as_double((long long)k); }
-};
+// Barycentrics (v of b, w of c) of the point of the triangle (0, b, c) closest
+// to P, by the same region tests as closest_tri with the dot products
+// relative to vertex a: bp = P - b and cp = P - c enter through
+// ab . bp = ab . P - ab . ab and so on.
+template <typename R>
+__device__ __forceinline__ void closest_rel(const R P[3], const R b[3], const R c[3], R bb, R bc, R cc, R& v, R& w) {
+    const R d1 = b[0] * P[0] + b[1] * P[1] + b[2] * P[2];
+    const R d2 = c[0] * P[0] + c[1] * P[1] + c[2] * P[2];
+    if (d1 <= (R)0 && d2 <= (R)0) { v = 0; w = 0; return; }
+    const R d3 = d1 - bb, d4 = d2 - bc, d5 = d1 - bc, d6 = d2 - cc;
+    if (d3 >= (R)0 && d4 <= d3) { v = 1; w = 0; return; }
+    if (d6 >= (R)0 && d5 <= d6) { v = 0; w = 1; return; }
+    const R vc = d1 * d4 - d3 * d2;
+    const R vb = d5 * d2 - d1 * d6;
+    const R va = d3 * d6 - d5 * d4;
+    // one division for all remaining regions: an edge's or the face's parameter
+    const bool e_ab = vc <= (R)0 && d1 >= (R)0 && d3 <= (R)0;
+    const bool e_ac = !e_ab && vb <= (R)0 && d2 >= (R)0 && d6 <= (R)0;
+    const bool e_bc = !e_ab && !e_ac && va <= (R)0 && (d4 - d3) >= (R)0 && (d5 - d6) >= (R)0;
+    const R den = e_ab ? d1 - d3 : e_ac ? d2 - d6 : e_bc ? (d4 - d3) + (d5 - d6) : va + vb + vc;
+    const R q = (R)1 / den;
+    if (e_ab) { v = d1 * q; w = 0; }
+    else if (e_ac) { v = 0; w = d2 * q; }
+    else if (e_bc) { w = (d4 - d3) * q; v = (R)1 - w; }
+    else { v = vb * q; w = vc * q; }
+}
+
+// Box and pair-test geometry of triangle t, axis r = 0..2 by lanes 4 q + r of
+// a warp (lane 4 q + 3 only takes part in the shuffles): the FP64 chain of a
+// lane is a third of a triangle's. ok: t is a triangle of the mesh. (The node
+// positions come from the wing frame: other threads of the launch write xg.)
+template <typename T>
+__device__ __forceinline__ void tri_setup(const MaskWs& m, const MaskArgs& a, int t, int r, bool ok, double reach) {
+    const unsigned all = 0xffffffffu;
+    const int ax = r < 3 ? r : 0, l0 = (threadIdx.x & 31) & ~3;
+    int id[3] = {0, 0, 0};
+    bool good = ok;
+    if (ok) {
+        for (int v = 0; v < 3; ++v) {
+            id[v] = a.tri[3 * t + v];
+            good = good && id[v] >= 0 && id[v] < a.n_nodes;
+        }
+        if (!good) m.cnt[4] = 1;
+    }
+    double X[3] = {0.0, 0.0, 0.0};
+    if (good)
+        for (int v = 0; v < 3; ++v) {
+            const double* x = a.xw + 3 * (size_t)id[v];
+            double s = a.XO[ax];
+            for (int c = 0; c < 3; ++c) s += a.R[3 * ax + c] * x[c];
+            X[v] = s;
+        }
+    const double b = X[1] - X[0], c = X[2] - X[0];
+    const T tb = (T)b, tc = (T)c;
+    // edge components of all three axes from the lanes of this triangle
+    T vb[3], vc[3];
+    for (int q = 0; q < 3; ++q) {
+        vb[q] = __shfl_sync(all, tb, l0 + q);
+        vc[q] = __shfl_sync(all, tc, l0 + q);
+    }
+    if (!ok || r == 3) return;
+    TriGeo<T>& g = *reinterpret_cast<TriGeo<T>*>(m.geo + (size_t)t * kTriGeoBytes);
+    int i0 = 0, e = 0, ca = 0;
+    T f = (T)0;
+    if (good) {
+        double l = ceil((fmin(X[0], fmin(X[1], X[2])) - reach) * a.inv_dx);
+        double h = floor((fmax(X[0], fmax(X[1], X[2])) + reach) * a.inv_dx);
+        l = fmax(l, ax == 0 ? (double)a.x_lo : 0.0);
+        h = fmin(h, ax == 0 ? (double)(a.x_hi - 1) : (double)((ax == 2 ? a.nz : a.n) - 1));
+        i0 = (int)l;
+        e = h >= l ? (int)(h - l) + 1 : 0;
+        const double cr = floor(X[0] * a.inv_dx);
+        ca = (int)cr;
+        f = (T)(X[0] - cr * a.dx);
+    }
+    g.i0[r] = i0;
+    g.e[r] = e;
+    g.ca[r] = ca;
+    g.f[r] = f;
+    g.b[r] = tb;
+    g.c[r] = tc;
+    g.m[r] = ((float)b + (float)c) * (1.0f / 3.0f);
+    if (r == 0) {
+        g.bb = vb[0] * vb[0] + vb[1] * vb[1] + vb[2] * vb[2];
+    } else if (r == 1) {
+        g.bc = vb[0] * vc[0] + vb[1] * vc[1] + vb[2] * vc[2];
+        // sphere about the centroid
+        float da = 0.0f, db = 0.0f, dc = 0.0f;
+        for (int q = 0; q < 3; ++q) {
+            const float fb = (float)vb[q], fc = (float)vc[q], mq = (fb + fc) * (1.0f / 3.0f);
+            da += mq * mq;
+            db += (fb - mq) * (fb - mq);
+            dc += (fc - mq) * (fc - mq);
+        }
+        g.r = sqrtf(fmaxf(da, fmaxf(db, dc))) * 1.00001f;
+    } else {
+        g.cc = vc[0] * vc[0] + vc[1] * vc[1] + vc[2] * vc[2];
+        if constexpr (sizeof(T) == 8) {   // unit normal (only the FP64 walks use it)
+            const float n[3] = {(float)(vb[1] * vc[2] - vb[2] * vc[1]), (float)(vb[2] * vc[0] - vb[0] * vc[2]),
+                                (float)(vb[0] * vc[1] - vb[1] * vc[0])};
+            // scaled by the largest component: no underflow of tiny areas' squares
+            const float big = fmaxf(fabsf(n[0]), fmaxf(fabsf(n[1]), fabsf(n[2])));
+            const float k = big > 0.0f ? 1.0f / big : 0.0f;
+            const float x = n[0] * k, y = n[1] * k, z = n[2] * k, len = x * x + y * y + z * z;
+            const float u = len >= 0.5f ? rsqrtf(len) : 0.0f;   // 0: degenerate (no area)
+            g.nrm[0] = x * u;
+            g.nrm[1] = y * u;
+            g.nrm[2] = z * u;
+        }
+    }
+}
 
 // First kernel of a call: zero chi/u_s and reset the key and winner of the
 // points the previous call touched (list `par`), clear the line flags
-// (n^2 bytes, 16-byte aligned), reset the other list's count, and the
-// global node positions X_O + R x^(w) (double).
-template <typename T>
-__global__ void k_mask_clear(MaskWs m, MaskArgs a, int par, T* chi, T* us, uint8_t* flag, size_t n3, size_t nflag) {
+// (n^2 bytes, 16-byte aligned), reset the other list's count, the global
+// node positions X_O + R x^(w) (double), and (BAND) the triangles' boxes and
+// geometry. The triangles start at the last thread (four each) and the nodes
+// at the first, so that as few warps as possible have both FP64 chains.
+template <typename T, bool BAND>
+__global__ void k_mask_prepare(MaskWs m, MaskArgs a, int par, T* chi, T* us, uint8_t* flag, size_t n3, size_t nflag,
+                               double reach) {
     const unsigned long long tid = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned long long nth = (unsigned long long)gridDim.x * blockDim.x;
     if (tid == 0) m.cnt[par ^ 1] = 0;
@@ -175,11 +296,18 @@ __global__ void k_mask_clear(MaskWs m, MaskArgs a, int par, T* chi, T* us, uint8
             m.xg[3 * i + r] = s;
         }
     }
+    if constexpr (BAND) {
+        // thread u from the end: whole warps, four lanes per triangle
+        const unsigned long long w = (nth - 1 - tid) >> 5;
+        const unsigned long long t = 8 * w + ((threadIdx.x & 31) >> 2);
+        if (8 * w < (unsigned long long)a.n_tri)   // uniform in the warp
+            tri_setup<T>(m, a, (int)t, threadIdx.x & 3, t < (unsigned long long)a.n_tri, reach);
+    }
     uint4* f4 = reinterpret_cast<uint4*>(flag);
     for (unsigned long long i = tid; i < nflag / 16; i += nth) f4[i] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < nflag % 16) flag[nflag / 16 * 16 + tid] = 0;
     const unsigned long long cnt = m.cnt[par];
-    const uint32_t* L = m.list[par];
+    const uint32_t* L = par ? m.list[1] : m.list[0];
     for (unsigned long long i = tid; i < cnt; i += nth) {
         const uint32_t p = L[i];
         m.key[p] = ~0ull;
@@ -189,167 +317,136 @@ __global__ void k_mask_clear(MaskWs m, MaskArgs a, int par, T* chi, T* us, uint8
     }
 }
 
-// One thread per triangle: bounding box dilated by the reach, its point
-// count, and the pair-test geometry.
-template <typename T>
-__global__ void k_mask_tris(MaskWs m, MaskArgs a, double reach) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= a.n_tri) return;
-    int ok = 1;
-    int id[3];
-    double lo[3], hi[3];
-    for (int r = 0; r < 3; ++r) { lo[r] = 1e300; hi[r] = -1e300; }
-    for (int v = 0; v < 3; ++v) {
-        id[v] = a.tri[3 * t + v];
-        if (id[v] < 0 || id[v] >= a.n_nodes) { ok = 0; break; }
+// Tolerance of near-ties of squared distances (FP64): 4 units in the last
+// place of the distance (the same pair recomputed may round differently).
+__device__ __forceinline__ double tie_limit(double d2) { return d2 + (d2 * 1.8e-15 + 1e-300); }
+
+// Warp (t, part) of wpt per triangle: points 32 part .. 32 part + 31 of
+// triangle t's box, and on by 32 wpt.
+static constexpr int kPairThreads = 256;
+enum PairWalk { kPairOne, kPairBound, kPairLeast, kPairTies };
+template <typename T, int WALK>
+__global__ void __launch_bounds__(kPairThreads) k_mask_pairs(MaskWs m, MaskArgs a, int par, int wpt) {
+    const uint32_t warp = (blockIdx.x * (uint32_t)kPairThreads + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    const int t = (int)(warp / (uint32_t)wpt);
+    if (t >= a.n_tri) return;   // whole warps leave together
+    const TriGeo<T> g = *reinterpret_cast<const TriGeo<T>*>(m.geo + (size_t)t * kTriGeoBytes);
+    const uint32_t ej = (uint32_t)g.e[1], ek = (uint32_t)g.e[2], cnt = (uint32_t)g.e[0] * ej * ek;
+    const uint32_t l1 = 32u * (warp % (uint32_t)wpt), step = 32u * (uint32_t)wpt;
+    const double reach = a.tw + a.h;
+    uint32_t* const list = par ? m.list[1] : m.list[0];
+    auto place = [&](uint32_t l, int& i, int& j, int& k) {
+        const uint32_t q = l / ek;
+        k = g.i0[2] + (int)(l - q * ek);
+        i = (int)(q / ej);
+        j = g.i0[1] + (int)(q - (uint32_t)i * ej);
+        i += g.i0[0];
+    };
+    auto index = [&](int i, int j, int k) { return ((uint32_t)i * (uint32_t)a.n + (uint32_t)j) * (uint32_t)a.nz + (uint32_t)k; };
+    auto dist2 = [&](int i, int j, int k) -> T {
+        const T dx = (T)a.dx;
+        const T P[3] = {(T)(i - g.ca[0]) * dx - g.f[0], (T)(j - g.ca[1]) * dx - g.f[1], (T)(k - g.ca[2]) * dx - g.f[2]};
+        T v, w, s = (T)0;
+        closest_rel<T>(P, g.b, g.c, g.bb, g.bc, g.cc, v, w);
         for (int r = 0; r < 3; ++r) {
-            const double q = m.xg[3 * id[v] + r];
-            lo[r] = fmin(lo[r], q);
-            hi[r] = fmax(hi[r], q);
+            const T q = P[r] - v * g.b[r] - w * g.c[r];
+            s += q * q;
         }
-    }
-    int e[3] = {0, 0, 0}, i0[3] = {0, 0, 0};
-    TriGeo<T> gt;
-    for (int r = 0; r < 3; ++r) { gt.ca[r] = 0; gt.f[r] = gt.b[r] = gt.c[r] = (T)0; }
-    gt.ca[3] = 0;
-    if (ok) {
-        for (int r = 0; r < 3; ++r) {
-            double l = ceil((lo[r] - reach) / a.dx), h = floor((hi[r] + reach) / a.dx);
-            l = fmax(l, r == 0 ? (double)a.x_lo : 0.0);
-            h = fmin(h, r == 0 ? (double)(a.x_hi - 1) : (double)((r == 2 ? a.nz : a.n) - 1));
-            i0[r] = (int)l;
-            e[r] = h >= l ? (int)(h - l) + 1 : 0;
-            const double ar = m.xg[3 * id[0] + r];
-            const double cr = floor(ar / a.dx);
-            gt.ca[r] = (int)cr;
-            gt.f[r] = (T)(ar - cr * a.dx);
-            gt.b[r] = (T)(m.xg[3 * id[1] + r] - ar);
-            gt.c[r] = (T)(m.xg[3 * id[2] + r] - ar);
+        return s;
+    };
+    auto offer = [&](uint32_t p, unsigned long long key) {
+        if (atomicMin(&m.key[p], key) == ~0ull) list[atomicAdd(&m.cnt[par], 1ull)] = p;
+    };
+    if constexpr (WALK == kPairOne) {
+        const T reach2 = (T)(reach * reach);
+        for (uint32_t l = l1 + lane; l < cnt; l += step) {
+            int i, j, k;
+            place(l, i, j, k);
+            const T d2 = dist2(i, j, k);
+            if (d2 < reach2) offer(index(i, j, k), ((unsigned long long)__float_as_uint((float)d2) << 32) | (uint32_t)t);
         }
     } else {
-        m.cnt[4] = 1;
-    }
-    int* b = m.box + 8 * t;
-    b[0] = i0[0]; b[1] = i0[1]; b[2] = i0[2];
-    b[3] = e[0]; b[4] = e[1]; b[5] = e[2];
-    b[6] = e[0] * e[1] * e[2];
-    *reinterpret_cast<TriGeo<T>*>(m.geo + (size_t)t * kTriGeoBytes) = gt;
-}
-
-// One block of 1024 threads: exclusive prefix sum of the box point counts
-// (per-thread chunks, then a scan of the chunk totals by warp shuffles).
-__global__ void k_mask_prefix(MaskWs m, MaskArgs a) {
-    __shared__ unsigned long long wsum[32];
-    const int nt = a.n_tri;
-    const int per = (nt + blockDim.x - 1) / blockDim.x;
-    const int t0 = threadIdx.x * per, t1 = min(nt, t0 + per);
-    unsigned long long local = 0;
-    for (int t = t0; t < t1; ++t) local += (unsigned long long)m.box[8 * t + 6];
-    // inclusive scan within the warp, then of the warp totals
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    unsigned long long inc = local;
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long v = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += v;
-    }
-    if (lane == 31) wsum[wid] = inc;
-    __syncthreads();
-    if (wid == 0) {
-        unsigned long long w = lane < (int)(blockDim.x >> 5) ? wsum[lane] : 0ull;
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long v = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += v;
+        // FP32 bounds of a pair's distance: the triangle lies in the disc of
+        // radius r about m in its plane (a ball if it has no normal), and a
+        // point of it with clamped barycentrics is at least as far as the
+        // closest one. Both are rounded outwards by err, ten times the
+        // rounding of coordinates of this size.
+        const float fdx = (float)a.dx, freach = (float)reach, err = 1e-5f * (g.r + freach);
+        const float ff[3] = {(float)g.f[0], (float)g.f[1], (float)g.f[2]};
+        auto at = [&](int i, int j, int k, float* P) {
+            P[0] = (float)(i - g.ca[0]) * fdx - ff[0];
+            P[1] = (float)(j - g.ca[1]) * fdx - ff[1];
+            P[2] = (float)(k - g.ca[2]) * fdx - ff[2];
+        };
+        auto lower = [&](const float* P) {
+            const float x = P[0] - g.m[0], y = P[1] - g.m[1], z = P[2] - g.m[2];
+            const float h = x * g.nrm[0] + y * g.nrm[1] + z * g.nrm[2], h2 = h * h;
+            const float in = fmaxf(sqrtf(fmaxf(x * x + y * y + z * z - h2, 0.0f)) - g.r - err, 0.0f);
+            return fmaxf(sqrtf(h2 + in * in) - err, 0.0f);
+        };
+        if constexpr (WALK == kPairBound) {
+            const float b[3] = {(float)g.b[0], (float)g.b[1], (float)g.b[2]}, c[3] = {(float)g.c[0], (float)g.c[1], (float)g.c[2]};
+            for (uint32_t l = l1 + lane; l < cnt; l += step) {
+                int i, j, k;
+                place(l, i, j, k);
+                float P[3], v, w, s = 0.0f;
+                at(i, j, k, P);
+                if (lower(P) > freach) continue;
+                closest_rel<float>(P, b, c, (float)g.bb, (float)g.bc, (float)g.cc, v, w);
+                v = fminf(fmaxf(v, 0.0f), 1.0f);
+                w = fminf(fmaxf(w, 0.0f), 1.0f - v);
+                for (int r = 0; r < 3; ++r) {
+                    const float q = P[r] - v * b[r] - w * c[r];
+                    s += q * q;
+                }
+                const double up = (double)(sqrtf(s) + err);
+                offer(index(i, j, k), (unsigned long long)__double_as_longlong(up * up));
+            }
+        } else {
+            const double reach2 = reach * reach;
+            // pairs that the bounds leave wait in the warp's queue until 32 are there
+            __shared__ uint32_t queue[kPairThreads / 32][64];
+            uint32_t* const Q = queue[threadIdx.x >> 5];
+            int nq = 0;
+            auto test = [&](bool on, uint32_t l) {
+                if (!on) return;
+                int i, j, k;
+                place(l, i, j, k);
+                const uint32_t p = index(i, j, k);
+                const double d2 = (double)dist2(i, j, k);
+                if (!(d2 < reach2)) return;
+                if constexpr (WALK == kPairTies) {
+                    if (d2 <= tie_limit(__longlong_as_double((long long)m.key[p]))) atomicMin(&m.win[p], t);
+                } else {
+                    atomicMin(&m.key[p], (unsigned long long)__double_as_longlong(d2));
+                }
+            };
+            for (uint32_t l0 = l1; l0 < cnt; l0 += step) {
+                const uint32_t l = l0 + lane;
+                bool in = l < cnt;
+                if (in) {
+                    int i, j, k;
+                    place(l, i, j, k);
+                    float P[3];
+                    at(i, j, k, P);
+                    const float lo = lower(P);
+                    // at most the least distance so far, with the tie's margin
+                    const unsigned long long key = __ldcg(&m.key[index(i, j, k)]);
+                    in = lo <= freach && lo * lo <= (float)__longlong_as_double((long long)key) * 1.0001f;
+                }
+                const unsigned b = __ballot_sync(0xffffffffu, in);
+                if (in) Q[nq + __popc(b & ((1u << lane) - 1u))] = l;
+                nq += __popc(b);
+                __syncwarp();
+                if (nq >= 32) {
+                    nq -= 32;
+                    test(true, Q[nq + lane]);
+                    __syncwarp();
+                }
+            }
+            test(lane < nq, lane < nq ? Q[lane] : 0u);
         }
-        wsum[lane] = w;   // inclusive totals of warps 0..lane
-    }
-    __syncthreads();
-    unsigned long long run = inc - local + (wid > 0 ? wsum[wid - 1] : 0ull);
-    if (threadIdx.x == blockDim.x - 1) {
-        m.cnt[2] = run + local;
-        m.pre[nt] = run + local;
-    }
-    for (int t = t0; t < t1; ++t) {
-        m.pre[t] = run;
-        run += (unsigned long long)m.box[8 * t + 6];
-    }
-}
-
-__device__ __forceinline__ int find_tri(const unsigned long long* pre, int nt, unsigned long long w) {
-    int lo = 0, hi = nt;  // pre[lo] <= w < pre[hi]
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (pre[mid] <= w) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
-template <typename T>
-__device__ __forceinline__ bool pair_dist(const MaskWs& m, const MaskArgs& a, int t, unsigned long long local,
-                                          uint32_t* pt, T* dist) {
-    const int* b = m.box + 8 * t;
-    const uint32_t l = (uint32_t)local, ek = (uint32_t)b[5], ej = (uint32_t)b[4];
-    const uint32_t q = l / ek;
-    const int k = b[2] + (int)(l - q * ek);
-    const int j = b[1] + (int)(q % ej);
-    const int i = b[0] + (int)(q / ej);
-    const TriGeo<T>& g = *reinterpret_cast<const TriGeo<T>*>(m.geo + (size_t)t * kTriGeoBytes);
-    // grid point minus vertex a, from whole cells and the vertex offset
-    const T dx = (T)a.dx;
-    T P[3] = {(T)(i - g.ca[0]) * dx - g.f[0], (T)(j - g.ca[1]) * dx - g.f[1], (T)(k - g.ca[2]) * dx - g.f[2]};
-    T A0[3] = {(T)0, (T)0, (T)0};
-    T B0[3] = {g.b[0], g.b[1], g.b[2]};
-    T C0[3] = {g.c[0], g.c[1], g.c[2]};
-    T bary[3];
-    const T d = sqrt(closest_tri<T>(P, A0, B0, C0, bary));
-    *pt = (uint32_t)(((size_t)i * a.n + j) * a.nz + k);
-    *dist = d;
-    return d < (T)(a.tw + a.h);
-}
-
-template <typename T>
-__global__ void k_mask_scatter1(MaskWs m, MaskArgs a, int par) {
-    const unsigned long long W = m.cnt[2];
-    for (unsigned long long w = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; w < W;
-         w += (unsigned long long)gridDim.x * blockDim.x) {
-        const int t = find_tri(m.pre, a.n_tri, w);
-        uint32_t p;
-        T d;
-        if (!pair_dist<T>(m, a, t, w - m.pre[t], &p, &d)) continue;
-        // FP32: distance bits above the triangle index, so the minimum key
-        // also holds the winner (exact ties -> smallest index); FP64: the
-        // distance alone, the winner by k_mask_scatter2
-        unsigned long long key = KeyBits<T>::of(d);
-        if constexpr (sizeof(T) == 4) key = (key << 32) | (unsigned long long)(uint32_t)t;
-        const unsigned long long old = atomicMin(&m.key[p], key);
-        if (old == ~0ull) {
-            const unsigned long long slot = atomicAdd(&m.cnt[par], 1ull);
-            m.list[par][slot] = p;
-        }
-    }
-}
-
-// Pairs within a few units in the last place of the minimum (the same
-// distance recomputed here may round differently from the first pass):
-// smallest triangle index wins, so near-exact ties go to the smaller index.
-template <typename T> struct Ulps;
-template <> struct Ulps<float> {
-    static __device__ __forceinline__ float of(float d) { return d * 4.8e-7f + 1e-30f; }
-};
-template <> struct Ulps<double> {
-    static __device__ __forceinline__ double of(double d) { return d * 9.0e-16 + 1e-300; }
-};
-
-template <typename T>
-__global__ void k_mask_scatter2(MaskWs m, MaskArgs a) {
-    const unsigned long long W = m.cnt[2];
-    for (unsigned long long w = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; w < W;
-         w += (unsigned long long)gridDim.x * blockDim.x) {
-        const int t = find_tri(m.pre, a.n_tri, w);
-        uint32_t p;
-        T d;
-        if (!pair_dist<T>(m, a, t, w - m.pre[t], &p, &d)) continue;
-        const T dmin = KeyBits<T>::val(m.key[p]);
-        if (d <= dmin + Ulps<T>::of(dmin)) atomicMin(&m.win[p], t);
     }
 }
 
@@ -357,48 +454,62 @@ __device__ __forceinline__ double chi_profile(double d, double tw, double h, int
     if (profile == 1) return 0.5 * (1.0 - tanh((d - tw) / h));
     if (d <= tw - h) return 1.0;
     if (d >= tw + h) return 0.0;
-    return 0.5 * (1.0 + cos(M_PI * (d - tw + h) / (2.0 * h)));
+    return 0.5 * (1.0 + cospi((d - tw + h) * (0.5 / h)));
 }
 
 // chi and u_s at grid point p from triangle t (double throughout).
 template <typename T>
 __device__ __forceinline__ void eval_point(const MaskWs& m, const MaskArgs& a, uint32_t p, int t, T* chi, T* us,
                                            uint8_t* flag) {
-    const size_t n = a.n, nz = a.nz, n3 = n * n * nz;
-    const int k = (int)(p % nz), j = (int)((p / nz) % n), i = (int)(p / (n * nz));
-    const double X[3] = {i * a.dx, j * a.dx, k * a.dx};
+    const uint32_t un = (uint32_t)a.n, unz = (uint32_t)a.nz;
+    const size_t n3 = (size_t)un * un * unz;
+    const uint32_t line = p / unz, i = line / un;
+    const int k = (int)(p - line * unz), j = (int)(line - i * un);
     const int id[3] = {a.tri[3 * t], a.tri[3 * t + 1], a.tri[3 * t + 2]};
-    double P[3], V[3][3];
-    for (int v = 0; v < 3; ++v)
-        for (int r = 0; r < 3; ++r) V[v][r] = m.xg[3 * id[v] + r] - m.xg[3 * id[0] + r];
-    for (int r = 0; r < 3; ++r) P[r] = X[r] - m.xg[3 * id[0] + r];
-    double bary[3];
-    const double d = sqrt(closest_tri<double>(P, V[0], V[1], V[2], bary));
-    const double c = chi_profile(d, a.tw, a.h, a.profile);
-    chi[p] = (T)c;
-    if (c > 0.0 || a.profile == 1) {
-        double vl[3] = {0, 0, 0};
-        for (int v = 0; v < 3; ++v)
-            for (int r = 0; r < 3; ++r) vl[r] += bary[v] * a.vw[3 * id[v] + r];
-        double rr[3];
-        for (int r = 0; r < 3; ++r) rr[r] = X[r] - a.XO[r];
+    const double X[3] = {(int)i * a.dx, j * a.dx, k * a.dx};
+    double P[3], b[3], c[3], bb = 0.0, bc = 0.0, cc = 0.0;
+    for (int r = 0; r < 3; ++r) {
+        const double x0 = m.xg[3 * id[0] + r];
+        P[r] = X[r] - x0;
+        b[r] = m.xg[3 * id[1] + r] - x0;
+        c[r] = m.xg[3 * id[2] + r] - x0;
+        bb += b[r] * b[r];
+        bc += b[r] * c[r];
+        cc += c[r] * c[r];
+    }
+    double v, w, d2 = 0.0;
+    closest_rel<double>(P, b, c, bb, bc, cc, v, w);
+    for (int r = 0; r < 3; ++r) {
+        const double q = P[r] - v * b[r] - w * c[r];
+        d2 += q * q;
+    }
+    const double chi_p = chi_profile(sqrt(d2), a.tw, a.h, a.profile);
+    chi[p] = (T)chi_p;
+    if (chi_p > 0.0 || a.profile == 1) {
+        const double u = 1.0 - v - w;
+        double vl[3], rr[3];
+        for (int r = 0; r < 3; ++r) {
+            vl[r] = u * a.vw[3 * id[0] + r] + v * a.vw[3 * id[1] + r] + w * a.vw[3 * id[2] + r];
+            rr[r] = X[r] - a.XO[r];
+        }
         const double rot[3] = {a.Om[1] * rr[2] - a.Om[2] * rr[1], a.Om[2] * rr[0] - a.Om[0] * rr[2],
                                a.Om[0] * rr[1] - a.Om[1] * rr[0]};
         for (int r = 0; r < 3; ++r) {
             double g = a.VO[r] + rot[r];
-            for (int cc = 0; cc < 3; ++cc) g += a.R[3 * r + cc] * vl[cc];
+            for (int q = 0; q < 3; ++q) g += a.R[3 * r + q] * vl[q];
             us[r * n3 + p] = (T)g;
         }
-        if (c > 0.0) flag[(size_t)i * n + j] = 1;
+        if (chi_p > 0.0) flag[line] = 1;
     }
 }
 
 template <typename T>
 __global__ void k_mask_eval(MaskWs m, MaskArgs a, int par, T* chi, T* us, uint8_t* flag) {
     const unsigned long long cnt = m.cnt[par];
+    const uint32_t* const list = par ? m.list[1] : m.list[0];
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
          i += (unsigned long long)gridDim.x * blockDim.x) {
-        const uint32_t p = m.list[par][i];
+        const uint32_t p = list[i];
         int t;
         if constexpr (sizeof(T) == 4) {   // the winner is the key's low word; kept for the VJP
             t = (int)(uint32_t)m.key[p];
