@@ -44,6 +44,7 @@ struct ps_ctx {
     CUtensorMap tmU, tmA5;    // TMA descriptors of the x passes' inputs
     CUtensorMap tmG;          // adjoint G (x-inverse input), with_adjoint only
     CUtensorMap tmUp, tmHp;   // U and H in x-forward boxes (L2 prefetch)
+    CUtensorMap tmP;          // the pressure's Pi_hat in field 3 of A (x-inverse input)
     CUtensorMap tmN;          // keep_uw: the pressure's N fields (y-forward input)
     bool uw_valid;            // keep_uw: B holds u and omega of the current state
     // adjoint (with_adjoint): lam, mu, G, W, Ub, Wb spectral; u, w, nb physical
@@ -625,6 +626,8 @@ ps_status ps_init(const ps_params* p, void* cuda_stream, void* workspace_dev, si
             !encode_rows(&c->tmB, c->b.B, c->fp64, (size_t)6 * n * n, kp.Kzp, ops->cy4, ops->br4) ||
             !encode_rows(&c->tmU, c->b.U, c->fp64, (size_t)3 * Kk * Kk, kp.Kzp, ops->cx1, ops->br2) ||
             !encode_rows(&c->tmA5, c->b.A, c->fp64, (size_t)6 * Kk * n, kp.Kzp, ops->cx5, ops->br4) ||
+            !encode_rows(&c->tmP, w + L.A + (size_t)3 * n * Kk * kp.Kzp * 2 * c->elem, c->fp64, (size_t)Kk * Kk, kp.Kzp,
+                         ops->cx1, ops->br2) ||
             !encode_rows(&c->tmUp, c->b.U, c->fp64, (size_t)3 * Kk * Kk, kp.Kzp, ops->cx5, ops->br2) ||
             !encode_rows(&c->tmHp, c->b.H, c->fp64, (size_t)3 * Kk * Kk, kp.Kzp, ops->cx5, ops->br2)) {
             delete c;
@@ -634,6 +637,7 @@ ps_status ps_init(const ps_params* p, void* cuda_stream, void* workspace_dev, si
         c->b.tmB = &c->tmB;
         c->b.tmU = &c->tmU;
         c->b.tmA5 = &c->tmA5;
+        c->b.tmP = &c->tmP;
         c->b.tmUp = &c->tmUp;
         c->b.tmHp = &c->tmHp;
         c->b.tmG = nullptr;

@@ -23,6 +23,7 @@ struct Bufs {
     const CUtensorMap* tmB;  // B as rows of 2 Kzp reals (y-forward input)
     const CUtensorMap* tmU;  // U as rows of 2 Kzp reals (x-inverse input)
     const CUtensorMap* tmA5; // A as rows of 2 Kzp reals (x-forward input)
+    const CUtensorMap* tmP;  // field 3 of A as K K rows of 2 Kzp reals (the pressure's Pi_hat, x-inverse input)
     const CUtensorMap* tmUp; // U, H as rows of 2 Kzp reals, x-forward box (L2 prefetch)
     const CUtensorMap* tmHp;
     const CUtensorMap* tmG;  // adjoint G as rows of 2 Kzp reals, x-inverse box (null without adjoint)
@@ -35,7 +36,7 @@ struct Bufs {
 static constexpr int kEvPerStep = 10;
 
 struct Ops {
-    int n, nz, C, C5, G;
+    int n, nz, G;
     int cy2, br2, cy4, br4;   // TMA box widths (complex) and heights of the y passes
     int cx1, cx5;             // TMA box widths of the x passes (heights br2, br4)
     int zblocks;  // blocks of the z pass (= number of force partials), set by prepare
@@ -44,9 +45,8 @@ struct Ops {
     cudaError_t (*step)(const KP&, const Bufs&, int first, int resume, cudaStream_t, cudaEvent_t* ev);
     cudaError_t (*set_velocity)(const KP&, const Bufs&, const void* u, cudaStream_t);
     cudaError_t (*get_velocity)(const KP&, const Bufs&, void* u, cudaStream_t);
-    // generic 3-field transforms between compact spectral arrays (3 x
-    // [ky][kx][kz]) and physical arrays (3 x n^3); A, B are used as scratch
-    cudaError_t (*inv3)(const KP&, const Bufs&, const void* spec, void* phys, cudaStream_t);
+    // forward transform of 3 physical fields (3 x n^2 nz) to a compact spectral
+    // array (3 x [ky][kx][kz]); A, B are used as scratch
     cudaError_t (*fwd3)(const KP&, const Bufs&, const void* phys, void* spec, cudaStream_t);
     // physical u and omega of the state in U (A, B used as scratch)
     cudaError_t (*inv_uw)(const KP&, const Bufs&, void* u, void* w, cudaStream_t);
@@ -70,12 +70,7 @@ template <typename T, int N, int NZ = N> struct Engine {
     using GE = Geo<T, N>;
     using GZ = Geo<T, NZ>;
     static constexpr int KZ_ = GZ::KZP;   // kz columns (compile-time in the x/y passes)
-    static constexpr size_t tw_bytes = (size_t)GE::tw_n * sizeof(C2);
-    static constexpr size_t sm_strided = tw_bytes + (size_t)N * GE::C * sizeof(C2);
-    static constexpr size_t sm_x5 = tw_bytes + (size_t)3 * N * GE::C5 * sizeof(C2);
     static constexpr size_t sm_zp = (size_t)GZ::zsmem(GZ::LZ);
-    static constexpr int thr_s = GE::C * GE::G;
-    static constexpr int thr_5 = GE::C5 * GE::G;
     static constexpr int thr_zp = 3 * GZ::LZ * GZ::G;
     // persistent physical <-> z-spectral transforms
     using ZP = ZPhys<T, NZ>;
@@ -124,6 +119,10 @@ template <typename T, int N, int NZ = N> struct Engine {
         static int g = 0;
         return g;
     }
+    static int& x1pgrid() {   // plain x-inverse (no curl)
+        static int g = 0;
+        return g;
+    }
     static int& x5grid() {
         static int g = 0;
         return g;
@@ -144,21 +143,11 @@ template <typename T, int N, int NZ = N> struct Engine {
 
     static cudaError_t prepare(int nsm, int* zb) {
         cudaError_t e;
-        if ((e = attr(k_xinv<T, N, 6>, sm_strided))) return e;
-        if ((e = attr(k_xinv<T, N, 3>, sm_strided))) return e;
-        if ((e = attr(k_yinv<T, N, 6>, sm_strided))) return e;
-        if ((e = attr(k_yinv<T, N, 3>, sm_strided))) return e;
-        if ((e = attr(k_yfwd<T, N>, sm_strided))) return e;
         if ((e = attr(k_zpass<T, NZ, false, false, N>, sm_zp))) return e;
         if ((e = attr(k_zpass<T, NZ, true, false, N>, sm_zp))) return e;
-        if ((e = attr(k_xinv<T, N, 1>, sm_strided))) return e;
-        if ((e = attr(k_yinv<T, N, 1>, sm_strided))) return e;
         if ((e = attr(k_zinv_sub<T, NZ>, sm_zs))) return e;
         if ((e = attr(k_zfwd_phys<T, NZ>, sm_zf))) return e;
         if ((e = attr(k_zinv_phys<T, NZ>, sm_zi))) return e;
-        if ((e = attr(k_xfwd<T, N, 0>, sm_x5))) return e;
-        if ((e = attr(k_xfwd<T, N, 1>, sm_x5))) return e;
-        if ((e = attr(k_xfwd<T, N, 2>, sm_x5))) return e;
         int occ = 0;
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_zpass<T, NZ, false, false, N>, thr_zp, sm_zp))) return e;
         if (occ < 1) occ = 1;
@@ -174,6 +163,7 @@ template <typename T, int N, int NZ = N> struct Engine {
         y4grid() = nsm * (occ < 1 ? 1 : occ);
         if ((e = attr(k_xinv_tma<T, N, 6, KZ_>, sm_x1))) return e;
         if ((e = attr(k_xinv_tma<T, N, 3, KZ_>, sm_x1))) return e;
+        if ((e = attr(k_xinv_tma<T, N, 1, KZ_>, sm_x1))) return e;
         if ((e = attr(k_yinv_tma<T, N, 3, KZ_>, sm_y2))) return e;
         if ((e = attr(k_yinv_tma<T, N, 1, KZ_>, sm_y2))) return e;
         if ((e = attr(k_xfwd_tma<T, N, 0, false, KZ_>, sm_x5t))) return e;
@@ -188,6 +178,8 @@ template <typename T, int N, int NZ = N> struct Engine {
         x5sgrid() = nsm * (occ < 1 ? 1 : occ);
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xinv_tma<T, N, 6, KZ_>, thr_x1, sm_x1))) return e;
         x1grid() = nsm * (occ < 1 ? 1 : occ);
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xinv_tma<T, N, 3, KZ_>, thr_x1, sm_x1))) return e;
+        x1pgrid() = nsm * (occ < 1 ? 1 : occ);
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xfwd_tma<T, N, 0, false, KZ_>, thr_x5, sm_x5t))) return e;
         x5grid() = nsm * (occ < 1 ? 1 : occ);
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_zinv_phys<T, NZ>, thr_zi, sm_zi))) return e;
@@ -198,9 +190,6 @@ template <typename T, int N, int NZ = N> struct Engine {
         zsgrid() = nsm * (occ < 1 ? 1 : occ);
         return cudaSuccess;
     }
-
-    static dim3 grid_xs(const KP& kp, int C) { return dim3(kp.Kzp / C, kp.K); }
-    static dim3 grid_ys(const KP& kp) { return dim3(kp.Kzp / GE::C, N); }
 
 
     // resume: B already holds u and omega of the state (y-inverse output,
@@ -241,27 +230,28 @@ template <typename T, int N, int NZ = N> struct Engine {
 
     static cudaError_t set_velocity(const KP& kp, const Bufs& b, const void* u, cudaStream_t s) {
         const C2* tw = (const C2*)b.tw;
-        k_zfwd_phys<T, NZ><<<zfgrid(), thr_zf, sm_zf, s>>>(kp, (const T*)u, (C2*)b.B, twz(b.tw), b.err);
-        k_yfwd<T, N><<<grid_ys(kp), thr_s, sm_strided, s>>>(kp, (const C2*)b.B, (C2*)b.A, tw);
-        k_xfwd_tma<T, N, 1, false, KZ_><<<x5grid(), thr_x5, sm_x5t, s>>>(*b.tmA5, *b.tmUp, *b.tmHp, kp, (C2*)b.U, (C2*)b.H,
+        KP k1 = kp;
+        k1.xs0 = 0; k1.xsn = N; k1.part_off = 0;
+        k_zfwd_phys<T, NZ><<<zfgrid(), thr_zf, sm_zf, s>>>(k1, (const T*)u, (C2*)b.B, twz(b.tw), b.err);
+        k_yfwd_tma<T, N, GE::CY4, 3, KZ_><<<y4grid(), thr_y4, sm_y4, s>>>(*b.tmB, k1, (C2*)b.A, tw, b.err);
+        k_xfwd_tma<T, N, 1, false, KZ_><<<x5grid(), thr_x5, sm_x5t, s>>>(*b.tmA5, *b.tmUp, *b.tmHp, k1, (C2*)b.U, (C2*)b.H,
                                                             (const T*)b.Ex, (const T*)b.Ez, 0, tw, b.err);
         return cudaGetLastError();
     }
 
-    static cudaError_t get_velocity(const KP& kp, const Bufs& b, void* u, cudaStream_t s) {
+    // physical (3 x n^2 nz) inverse transform of the three spectral fields
+    // that tm maps (U, or the adjoint array G)
+    static cudaError_t inverse3(const KP& kp, const Bufs& b, const CUtensorMap& tm, void* phys, cudaStream_t s) {
         const C2* tw = (const C2*)b.tw;
-        k_xinv<T, N, 3><<<grid_xs(kp, GE::C), thr_s, sm_strided, s>>>(kp, (const C2*)b.U, (C2*)b.A, tw);
-        k_yinv<T, N, 3><<<grid_ys(kp), thr_s, sm_strided, s>>>(kp, (const C2*)b.A, (C2*)b.B, tw);
-        k_zinv_phys<T, NZ><<<zigrid(), thr_zi, sm_zi, s>>>(kp, (const C2*)b.B, (T*)u, twz(b.tw), b.err);
+        KP k1 = kp;
+        k1.xs0 = 0; k1.xsn = N; k1.part_off = 0;
+        k_xinv_tma<T, N, 3, KZ_><<<x1pgrid(), thr_x1, sm_x1, s>>>(tm, k1, (C2*)b.A, tw, b.err);
+        k_yinv_tma<T, N, 3, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, (C2*)b.B, tw, b.err);
+        k_zinv_phys<T, NZ><<<zigrid(), thr_zi, sm_zi, s>>>(k1, (const C2*)b.B, (T*)phys, twz(b.tw), b.err);
         return cudaGetLastError();
     }
-
-    static cudaError_t inv3(const KP& kp, const Bufs& b, const void* spec, void* phys, cudaStream_t s) {
-        const C2* tw = (const C2*)b.tw;
-        k_xinv<T, N, 3><<<grid_xs(kp, GE::C), thr_s, sm_strided, s>>>(kp, (const C2*)spec, (C2*)b.A, tw);
-        k_yinv<T, N, 3><<<grid_ys(kp), thr_s, sm_strided, s>>>(kp, (const C2*)b.A, (C2*)b.B, tw);
-        k_zinv_phys<T, NZ><<<zigrid(), thr_zi, sm_zi, s>>>(kp, (const C2*)b.B, (T*)phys, twz(b.tw), b.err);
-        return cudaGetLastError();
+    static cudaError_t get_velocity(const KP& kp, const Bufs& b, void* u, cudaStream_t s) {
+        return inverse3(kp, b, *b.tmU, u, s);
     }
 
     static cudaError_t fwd3(const KP& kp, const Bufs& b, const void* phys, void* spec, cudaStream_t s) {
@@ -275,16 +265,8 @@ template <typename T, int N, int NZ = N> struct Engine {
         return cudaGetLastError();
     }
 
-    // physical (3 x n^3) inverse transform of the adjoint array G (b.tmG)
-    // through the TMA x and y passes
     static cudaError_t inv_g(const KP& kp, const Bufs& b, void* phys, cudaStream_t s) {
-        const C2* tw = (const C2*)b.tw;
-        KP k1 = kp;
-        k1.xs0 = 0; k1.xsn = N; k1.part_off = 0;
-        k_xinv_tma<T, N, 3, KZ_><<<x1grid(), thr_x1, sm_x1, s>>>(*b.tmG, k1, (C2*)b.A, tw, b.err);
-        k_yinv_tma<T, N, 3, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, (C2*)b.B, tw, b.err);
-        k_zinv_phys<T, NZ><<<zigrid(), thr_zi, sm_zi, s>>>(k1, (const C2*)b.B, (T*)phys, twz(b.tw), b.err);
-        return cudaGetLastError();
+        return inverse3(kp, b, *b.tmG, phys, s);
     }
 
     // static pressure p = Pi - (1/2)|u|^2 of the state U with the current
@@ -312,7 +294,7 @@ template <typename T, int N, int NZ = N> struct Engine {
         C2* pih = (C2*)b.A + (size_t)3 * N * GE::K * kp.Kzp;
         k_xfwd_tma<T, N, 3, false, KZ_><<<x5grid(), thr_x5, sm_x5t, s>>>(*b.tmA5, *b.tmUp, *b.tmHp, k1, pih, nullptr,
                                                             (const T*)b.Ex, (const T*)b.Ez, 0, tw, b.err);
-        k_xinv<T, N, 1><<<grid_xs(k1, GE::C), thr_s, sm_strided, s>>>(k1, pih, (C2*)b.A, tw);
+        k_xinv_tma<T, N, 1, KZ_><<<x1pgrid(), thr_x1, sm_x1, s>>>(*b.tmP, k1, (C2*)b.A, tw, b.err);
         k_yinv_tma<T, N, 1, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, nout, tw, b.err);
         k_zinv_sub<T, NZ><<<zsgrid(), thr_zs, sm_zs, s>>>(k1, (const C2*)nout, (T*)p, twz(b.tw), b.err);
         return cudaGetLastError();
@@ -351,7 +333,7 @@ template <typename T, int N, int NZ = N> struct Engine {
 
     static Ops ops() {
         Ops o;
-        o.n = N; o.nz = NZ; o.C = GE::C; o.C5 = GE::C5; o.G = GE::G;
+        o.n = N; o.nz = NZ; o.G = GE::G;
         o.cy2 = GE::CY2; o.br2 = GE::brows(GE::K); o.cy4 = GE::CY4; o.br4 = GE::brows(N);
         o.cx1 = GE::CX1; o.cx5 = GE::CX5;
         o.zblocks = 0;
@@ -359,7 +341,6 @@ template <typename T, int N, int NZ = N> struct Engine {
         o.step = &step;
         o.set_velocity = &set_velocity;
         o.get_velocity = &get_velocity;
-        o.inv3 = &inv3;
         o.fwd3 = &fwd3;
         o.inv_uw = &inv_uw;
         o.inv_g = &inv_g;

@@ -26,9 +26,9 @@
 //
 // Pass order of a step (P = Leray projection, E = exp(-nu |k|^2 dt)); the
 // step uses the TMA-staged kernels k_xinv_tma, k_yinv_tma, k_zpass,
-// k_yfwd_tma, k_xfwd_tma; the plain kernels k_xinv/k_yinv/k_yfwd/k_xfwd and
-// the physical <-> z-spectral kernels serve ps_set/get_velocity and the
-// adjoint's generic transforms:
+// k_yfwd_tma, k_xfwd_tma; their plain 3-field (1-field) variants and the
+// physical <-> z-spectral kernels serve ps_set/get_velocity, the pressure and
+// the adjoint's transforms:
 //   1 x-inverse of u_hat and omega_hat = i k x u_hat (curl fused)    U -> A (6)
 //   2 y-inverse                                                      A -> B (6)
 //   3 z c2r, n = u x omega - (chi/eta)(u - u_s), force/moment partial
@@ -186,16 +186,12 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* out, double* 
     }
 }
 
-// Launch geometry per (T, n): tile width C of the strided passes (128-byte
-// rows), C5 of the x-forward/update pass (three tiles must fit), the z
-// pass's lines per batch and the TMA passes' tile widths.
+// Launch geometry per (T, n): the z pass's lines per batch and the TMA
+// passes' tile widths (at most CW complex, 128-byte rows).
 template <typename T, int N> struct Geo {
     using C2 = cplx<T>;
     static constexpr int G = LineFFT<T, N, 1>::G;
     static constexpr int CW = 128 / (int)sizeof(C2);     // 16 (float), 8 (double)
-    static constexpr int C = CW;
-    static constexpr int C5 = (3 * N * CW * (int)sizeof(C2) <= 110 * 1024) ? CW
-                            : (3 * N * (CW / 2) * (int)sizeof(C2) <= 150 * 1024) ? CW / 2 : CW / 4;
     static constexpr int LP = N + N / 16;                  // padded z line
     // kept z modes, padded to the tile width
     static constexpr int KZ = (N - 1) / 3 + 1;
@@ -494,91 +490,6 @@ __device__ __forceinline__ cplx<T>* load_tw_split(cplx<T>* tw, const cplx<T>* tw
 template <typename C2>
 __device__ __forceinline__ void load_tw(C2* s, const C2* g, int n) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) s[i] = g[i];
-}
-
-// ---------------------------------------------------------------- pass 1
-// x-inverse of the three velocity components and, if NF == 6, of the
-// vorticity omega_hat = i k x u_hat (components 3..5).
-template <typename T, int N, int NF>
-__global__ void __launch_bounds__(Geo<T, N>::C * Geo<T, N>::G)
-k_xinv(KP kp, const cplx<T>* __restrict__ U, cplx<T>* __restrict__ A, const cplx<T>* __restrict__ twg) {
-    using C2 = cplx<T>;
-    using GE = Geo<T, N>;
-    constexpr int C = GE::C, G = GE::G;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    C2* tw = reinterpret_cast<C2*>(smraw);
-    C2* tile = tw + GE::tw_n;
-    const int col = threadIdx.x % C, g = threadIdx.x / C;
-    const int cz = blockIdx.x * C + col;
-    const bool okz = cz < kp.Kz;
-    const int cy = blockIdx.y;
-    const int K = kp.K, mmax = kp.mmax, Kzp = kp.Kzp;
-    const T ks = (T)kp.ks;   // wavenumbers in T: no double arithmetic per element
-    const T ky = ks * (T)cmode_of(cy, mmax, K);
-    const T kz = (T)kp.ksz * (T)cz;
-    const size_t FS = (size_t)K * K * Kzp;
-    const size_t AS = (size_t)N * K * Kzp;
-    load_tw(tw, twg, GE::tw_n);
-    auto addr = [&](int p) { return p * C + col; };
-#pragma unroll 1
-    for (int f = 0; f < NF; ++f) {
-        __syncthreads();
-        auto load = [&](int q) -> C2 {
-            const int m = mode_of(q, N);
-            if (!okz || m > mmax || m < -mmax) return cmk<C2>((T)0, (T)0);
-            const size_t o = ((size_t)cy * K + cidx_of(m, K)) * Kzp + cz;
-            const T kx = ks * (T)m;
-            if (f < 3) return U[f * FS + o];
-            if (f == 3) {  // i (ky uz - kz uy)
-                C2 uy = U[FS + o], uz = U[2 * FS + o];
-                return cmk<C2>(-(ky * uz.y - kz * uy.y), ky * uz.x - kz * uy.x);
-            }
-            if (f == 4) {  // i (kz ux - kx uz)
-                C2 ux = U[o], uz = U[2 * FS + o];
-                return cmk<C2>(-(kz * ux.y - kx * uz.y), kz * ux.x - kx * uz.x);
-            }
-            C2 ux = U[o], uy = U[FS + o];  // i (kx uy - ky ux)
-            return cmk<C2>(-(kx * uy.y - ky * ux.y), kx * uy.x - ky * ux.x);
-        };
-        auto store = [&](int x, C2 v) {
-            if (okz) A[f * AS + GE::arow(x, cy) * Kzp + cz] = v;
-        };
-        LineFFT<T, N, 1>::template run<false>(tile, tw, addr, g, load, store);
-    }
-}
-
-// ---------------------------------------------------------------- pass 2
-template <typename T, int N, int NF>
-__global__ void __launch_bounds__(Geo<T, N>::C * Geo<T, N>::G)
-k_yinv(KP kp, const cplx<T>* __restrict__ A, cplx<T>* __restrict__ B, const cplx<T>* __restrict__ twg) {
-    using C2 = cplx<T>;
-    using GE = Geo<T, N>;
-    constexpr int C = GE::C;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    C2* tw = reinterpret_cast<C2*>(smraw);
-    C2* tile = tw + GE::tw_n;
-    const int col = threadIdx.x % C, g = threadIdx.x / C;
-    const int cz = blockIdx.x * C + col;
-    const bool okz = cz < kp.Kz;
-    const int x = blockIdx.y;
-    const int K = kp.K, mmax = kp.mmax, Kzp = kp.Kzp;
-    const size_t AS = (size_t)N * K * Kzp;
-    const size_t BS = (size_t)N * N * Kzp;
-    load_tw(tw, twg, GE::tw_n);
-    auto addr = [&](int p) { return p * C + col; };
-#pragma unroll 1
-    for (int f = 0; f < NF; ++f) {
-        __syncthreads();
-        auto load = [&](int q) -> C2 {
-            const int m = mode_of(q, N);
-            if (!okz || m > mmax || m < -mmax) return cmk<C2>((T)0, (T)0);
-            return A[f * AS + GE::arow(x, cidx_of(m, K)) * Kzp + cz];
-        };
-        auto store = [&](int y, C2 v) {
-            if (okz) B[f * BS + ((size_t)x * N + y) * Kzp + cz] = v;
-        };
-        LineFFT<T, N, 1>::template run<false>(tile, tw, addr, g, load, store);
-    }
 }
 
 // ---------------------------------------------------------------- pass 3
@@ -942,129 +853,6 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
     }
 }
 
-// ---------------------------------------------------------------- pass 4
-template <typename T, int N>
-__global__ void __launch_bounds__(Geo<T, N>::C * Geo<T, N>::G)
-k_yfwd(KP kp, const cplx<T>* __restrict__ B, cplx<T>* __restrict__ A, const cplx<T>* __restrict__ twg) {
-    using C2 = cplx<T>;
-    using GE = Geo<T, N>;
-    constexpr int C = GE::C;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    C2* tw = reinterpret_cast<C2*>(smraw);
-    C2* tile = tw + GE::tw_n;
-    const int col = threadIdx.x % C, g = threadIdx.x / C;
-    const int cz = blockIdx.x * C + col;
-    const bool okz = cz < kp.Kz;
-    const int x = blockIdx.y;
-    const int K = kp.K, mmax = kp.mmax, Kzp = kp.Kzp;
-    const size_t AS = (size_t)N * K * Kzp;
-    const size_t BS = (size_t)N * N * Kzp;
-    load_tw(tw, twg, GE::tw_n);
-    auto addr = [&](int p) { return p * C + col; };
-#pragma unroll 1
-    for (int f = 0; f < 3; ++f) {
-        __syncthreads();
-        auto load = [&](int y) -> C2 {
-            if (!okz) return cmk<C2>((T)0, (T)0);
-            return B[f * BS + ((size_t)x * N + y) * Kzp + cz];
-        };
-        auto store = [&](int q, C2 v) {
-            const int m = mode_of(q, N);
-            if (okz && m <= mmax && m >= -mmax) A[f * AS + GE::arow(x, cidx_of(m, K)) * Kzp + cz] = v;
-        };
-        LineFFT<T, N, -1>::template run<false>(tile, tw, addr, g, load, store);
-    }
-}
-
-// ---------------------------------------------------------------- pass 5
-// MODE 0: time step (Euler if first != 0, else AB2); MODE 1: set velocity
-// (project with the mean kept, history cleared); MODE 2: plain truncated
-// forward transform (times 1/n^3) into U, H untouched.
-template <typename T, int N, int MODE>
-__global__ void __launch_bounds__(Geo<T, N>::C5 * Geo<T, N>::G)
-k_xfwd(KP kp, const cplx<T>* __restrict__ A, cplx<T>* __restrict__ U, cplx<T>* __restrict__ H,
-       const T* __restrict__ Ex, const T* __restrict__ Ez, int first, const cplx<T>* __restrict__ twg) {
-    using C2 = cplx<T>;
-    using GE = Geo<T, N>;
-    constexpr int C = GE::C5;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    C2* tw = reinterpret_cast<C2*>(smraw);
-    C2* tiles = tw + GE::tw_n;
-    const int col = threadIdx.x % C, g = threadIdx.x / C;
-    const int cz0 = blockIdx.x * C;
-    const int cz = cz0 + col;
-    const bool okz = cz < kp.Kz;
-    const int cy = blockIdx.y;
-    const int K = kp.K, mmax = kp.mmax, Kzp = kp.Kzp;
-    const size_t AS = (size_t)N * K * Kzp;
-    const size_t FS = (size_t)K * K * Kzp;
-    load_tw(tw, twg, GE::tw_n);
-    auto addr = [&](int p) { return p * C + col; };
-#pragma unroll 1
-    for (int f = 0; f < 3; ++f) {
-        C2* tile = tiles + f * N * C;
-        __syncthreads();
-        auto load = [&](int x) -> C2 {
-            if (!okz) return cmk<C2>((T)0, (T)0);
-            return A[f * AS + GE::arow(x, cy) * Kzp + cz];
-        };
-        auto store = [&](int q, C2 v) { tile[addr(q)] = v; };
-        LineFFT<T, N, -1>::template run<false>(tile, tw, addr, g, load, store);
-    }
-    __syncthreads();
-    const T s = (T)kp.ks, sz = (T)kp.ksz;
-    const T my = (T)cmode_of(cy, mmax, K);
-    const T invn3 = (T)kp.invn3;
-    const T dt = (T)kp.dt;
-    const T ey = Ex[cy];
-    for (int idx = threadIdx.x; idx < K * C; idx += blockDim.x) {
-        const int cx = idx / C, c = idx % C;
-        const int czz = cz0 + c;
-        if (czz >= kp.Kz) continue;
-        const int mx = cmode_of(cx, mmax, K);
-        const int q = mx >= 0 ? mx : mx + N;
-        const int a = q * C + c;
-        C2 n0 = tiles[a], n1 = tiles[N * C + a], n2 = tiles[2 * N * C + a];
-        n0.x *= invn3; n0.y *= invn3;
-        n1.x *= invn3; n1.y *= invn3;
-        n2.x *= invn3; n2.y *= invn3;
-        const T kx = s * (T)mx, ky = s * my, kz = sz * (T)czz;
-        const T k2 = kx * kx + ky * ky + kz * kz;
-        const bool zero = (mx == 0 && cy == 0 && czz == 0);
-        const size_t o = ((size_t)cy * K + cx) * Kzp + czz;
-        if constexpr (MODE == 2) {   // plain truncated forward transform into U
-            U[o] = n0; U[FS + o] = n1; U[2 * FS + o] = n2;
-            continue;
-        }
-        if (!zero) {
-            const T ik2 = (T)1 / k2;
-            const T dr = (kx * n0.x + ky * n1.x + kz * n2.x) * ik2;
-            const T di = (kx * n0.y + ky * n1.y + kz * n2.y) * ik2;
-            n0.x -= kx * dr; n0.y -= kx * di;
-            n1.x -= ky * dr; n1.y -= ky * di;
-            n2.x -= kz * dr; n2.y -= kz * di;
-        } else if (MODE == 0 && !kp.mean_free) {
-            n0 = n1 = n2 = cmk<C2>((T)0, (T)0);
-        }
-        if constexpr (MODE == 1) {
-            U[o] = n0; U[FS + o] = n1; U[2 * FS + o] = n2;
-            const C2 z = cmk<C2>((T)0, (T)0);
-            H[o] = z; H[FS + o] = z; H[2 * FS + o] = z;
-        } else {
-            const T E = Ex[cx] * ey * Ez[czz];
-            C2 nn[3] = {n0, n1, n2};
-#pragma unroll
-            for (int f = 0; f < 3; ++f) {
-                const C2 uq = first ? U[f * FS + o] : H[f * FS + o];
-                C2 un, qn;
-                ab2_update(uq, nn[f], E, dt, first != 0, un, qn);
-                U[f * FS + o] = un;
-                H[f * FS + o] = qn;
-            }
-        }
-    }
-}
-
 // --------------------------------------------- TMA-staged y passes
 // Persistent blocks walk a list of items (x plane, kz tile of CT columns,
 // field); each item's input tile arrives by tiled TMA copies into one of two
@@ -1259,7 +1047,8 @@ k_yfwd_tma(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict__ 
 //   w_x = i (ky Uz - kz Uy),  w_y = i kz Ux - Dx Uz,  w_z = Dx Uy - i ky Ux;
 // a thread keeps its last-stage outputs of Ux and Uy in registers until the
 // transforms that need them. Inputs arrive field by field (x, y, z) by TMA.
-// NF = 3: the plain x-inverse of three fields (one transform each, no curl).
+// NF = 3, 1: the plain x-inverse of NF fields (one transform each, no curl;
+// without the two register sets three blocks fit where the curl has two).
 // tm: U (or the array being transformed) as 2-D rows of 2 Kzp reals, row
 // (f K + cy) K + cx.
 template <typename T, int N, int NF = 6, int KZP_ = Geo<T, N>::KZP>
@@ -1294,9 +1083,10 @@ k_xinv_tma(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict__ 
     }
     load_tw(tw, twg, GE::tw_n);
     __syncthreads();
-    // load L: tile iteration L / 3, field L % 3
+    constexpr int NI = NF == 6 ? 3 : NF;   // input fields
+    // load L: tile iteration L / NI, field L % NI
     auto issue = [&](int L) {  // one thread
-        const int t = blockIdx.x + (L / 3) * gridDim.x, f = L % 3, buf = L & 1;
+        const int t = blockIdx.x + (L / NI) * gridDim.x, f = L % NI, buf = L & 1;
         if (t >= NTILE) return;
         const int cy = kp.ky0 + t / NTZ, czt = t % NTZ;
         fence_proxy_async();
@@ -1317,8 +1107,8 @@ k_xinv_tma(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict__ 
         const T kz = ksz * (T)cz;
         C2* out = A + cz;   // + f AS + arow(x, cy) KZP
 #pragma unroll 1
-        for (int f = 0; f < 3; ++f) {
-            const int L = 3 * ti + f, buf = L & 1;
+        for (int f = 0; f < NI; ++f) {
+            const int L = NI * ti + f, buf = L & 1;
             if (threadIdx.x == 0) issue(L + 1);
             const bool ok = mbar_wait(&bar[buf], (uint32_t)((L >> 1) & 1));
             if (__syncthreads_or(!ok)) {
@@ -1344,7 +1134,7 @@ k_xinv_tma(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict__ 
                 };
                 auto store = [&](int slot, int x, C2 v) {
                     C2* o = out + GE::arow(x, cy) * KZP;
-                    if constexpr (NF == 3) {            // plain: field f only
+                    if constexpr (NF < 6) {             // plain: field f only
                         if (okz) o[f * AS] = v;
                         return;
                     }
