@@ -231,10 +231,10 @@ void host_tables(const ps_params* p, std::vector<unsigned char>& tw, std::vector
     const int n = p->n, nz = nz_of(p), mm = mmax_of(n), K = 2 * mm + 1, Kz = mmax_of(nz) + 1;
     std::vector<C2> t((size_t)3 * (n + nz), cmk<C2>((T)0, (T)0));
     // stage twiddles of a length-m line at offset `base`
-    auto line_table = [&](int m, size_t base) {
-        const int S = n_stages(m);
+    auto line_table = [&](int m, int rm, size_t base) {
+        const int S = n_stages(m, rm);
         for (int s = 1; s < S; ++s) {
-            const int r = radix_at(m, s), Ls = ls_at(m, s), o = tw_offset(m, s);
+            const int r = radix_at(m, s, rm), Ls = ls_at(m, s, rm), o = tw_offset(m, s, rm);
             for (int tt = 1; tt < r; ++tt)
                 for (int k = 0; k < Ls; ++k) {
                     double c, sn;
@@ -246,10 +246,11 @@ void host_tables(const ps_params* p, std::vector<unsigned char>& tw, std::vector
     // the table of length-m lines at `base`: the stage twiddles, then for
     // m = 3M the M-line table at base + m and e^{2 pi i b q/m} at base + 2m
     auto tables = [&](int m, size_t base) {
-        line_table(m, base);
+        const int rm = max_radix(sizeof(T) == 8, m);   // the split's sub-lines take the line's radix
+        line_table(m, rm, base);
         if (m % 3 == 0) {
             const int M = m / 3;
-            line_table(M, base + (size_t)m);
+            line_table(M, rm, base + (size_t)m);
             for (int b = 1; b <= 2; ++b)
                 for (int q = 0; q < M; ++q) {
                     double c, sn;

@@ -4,6 +4,11 @@
 #pragma once
 #include "ps_kernels.cuh"
 
+// x-inverse: at most this many (ky, kz tile) tiles take the split kernel
+#ifndef PS_XSPLIT_TILES
+#define PS_XSPLIT_TILES 152
+#endif
+
 namespace ps {
 
 struct Bufs {
@@ -119,6 +124,10 @@ template <typename T, int N, int NZ = N> struct Engine {
         static int g = 0;
         return g;
     }
+    static int& xsgrid() {
+        static int g = 0;
+        return g;
+    }
     static int& x1pgrid() {   // plain x-inverse (no curl)
         static int g = 0;
         return g;
@@ -135,6 +144,19 @@ template <typename T, int N, int NZ = N> struct Engine {
         return g;
     }
     static constexpr int thr_x1 = GE::CX1 * GE::G;
+    // fewer (ky, kz tile) tiles than a GB300 has SMs: one item per output field
+    static constexpr bool XSPLIT = GE::K * (KZ_ / GE::CX1) <= PS_XSPLIT_TILES;
+    // pass 1: x-inverse with the curl
+    static void x_inverse(const KP& kp, const Bufs& b, cudaStream_t s) {
+        const C2* tw = (const C2*)b.tw;
+        if constexpr (XSPLIT) {
+            const int items = kp.kyn * (KZ_ / GE::CX1) * 6;
+            k_xinv_split<T, N, KZ_><<<items < xsgrid() ? items : xsgrid(), thr_x1, sm_x1, s>>>(*b.tmU, kp, (C2*)b.A, tw,
+                                                                                              b.err);
+        } else {
+            k_xinv_tma<T, N, 6, KZ_><<<x1grid(), thr_x1, sm_x1, s>>>(*b.tmU, kp, (C2*)b.A, tw, b.err);
+        }
+    }
     static constexpr int thr_x5 = GE::CX5 * GE::G;
     static constexpr size_t sm_y2 = (size_t)GE::y2_smem(GE::CY2, GE::Y2NB);
     static constexpr size_t sm_y4 = (size_t)GE::y4_smem(GE::CY4);
@@ -162,6 +184,12 @@ template <typename T, int N, int NZ = N> struct Engine {
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_yfwd_tma<T, N, GE::CY4, 3, KZ_>, thr_y4, sm_y4))) return e;
         y4grid() = nsm * (occ < 1 ? 1 : occ);
         if ((e = attr(k_xinv_tma<T, N, 6, KZ_>, sm_x1))) return e;
+        if constexpr (XSPLIT) {
+            if ((e = attr(k_xinv_split<T, N, KZ_>, sm_x1))) return e;
+            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xinv_split<T, N, KZ_>, thr_x1, sm_x1)))
+                return e;
+            xsgrid() = nsm * (occ < 1 ? 1 : occ);
+        }
         if ((e = attr(k_xinv_tma<T, N, 3, KZ_>, sm_x1))) return e;
         if ((e = attr(k_xinv_tma<T, N, 1, KZ_>, sm_x1))) return e;
         if ((e = attr(k_yinv_tma<T, N, 3, KZ_>, sm_y2))) return e;
@@ -201,7 +229,7 @@ template <typename T, int N, int NZ = N> struct Engine {
         k1.xs0 = 0; k1.xsn = N; k1.part_off = 0;
         const bool sp = b.chi_sp != nullptr;   // sponge term: six-field z/y-forward variants
         if (ev) cudaEventRecord(ev[0], s);
-        if (!resume) k_xinv_tma<T, N, 6, KZ_><<<x1grid(), thr_x1, sm_x1, s>>>(*b.tmU, kp, (C2*)b.A, tw, b.err);
+        if (!resume) x_inverse(kp, b, s);
         if (ev) { cudaEventRecord(ev[1], s); cudaEventRecord(ev[2], s); }
         if (!resume) k_yinv_tma<T, N, 6, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, (C2*)b.B, tw, b.err);
         if (ev) { cudaEventRecord(ev[3], s); cudaEventRecord(ev[4], s); }
@@ -283,7 +311,7 @@ template <typename T, int N, int NZ = N> struct Engine {
         KP k1 = kp;
         k1.xs0 = 0; k1.xsn = N; k1.part_off = 0;
         if (!resume) {
-            k_xinv_tma<T, N, 6, KZ_><<<x1grid(), thr_x1, sm_x1, s>>>(*b.tmU, k1, (C2*)b.A, tw, b.err);
+            x_inverse(k1, b, s);
             k_yinv_tma<T, N, 6, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, (C2*)b.B, tw, b.err);
         }
         C2* nout = b.N3 ? (C2*)b.N3 : (C2*)b.B;
@@ -306,7 +334,7 @@ template <typename T, int N, int NZ = N> struct Engine {
         const C2* tw = (const C2*)b.tw;
         KP k1 = kp;
         k1.xs0 = 0; k1.xsn = N; k1.part_off = 0;
-        k_xinv_tma<T, N, 6, KZ_><<<x1grid(), thr_x1, sm_x1, s>>>(*b.tmU, k1, (C2*)b.A, tw, b.err);
+        x_inverse(k1, b, s);
         k_yinv_tma<T, N, 6, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, (C2*)b.B, tw, b.err);
         const size_t BS = (size_t)N * N * k1.Kzp;
         k_zinv_phys<T, NZ><<<zigrid(), thr_zi, sm_zi, s>>>(k1, (const C2*)b.B, (T*)u, twz(b.tw), b.err);
@@ -317,7 +345,7 @@ template <typename T, int N, int NZ = N> struct Engine {
     static cudaError_t slab_phase(const KP& kp, const Bufs& b, int phase, int first, cudaStream_t s) {
         const C2* tw = (const C2*)b.tw;
         if (phase == 0) {
-            k_xinv_tma<T, N, 6, KZ_><<<x1grid(), thr_x1, sm_x1, s>>>(*b.tmU, kp, (C2*)b.A, tw, b.err);
+            x_inverse(kp, b, s);
         } else if (phase == 1) {
             k_yinv_tma<T, N, 6, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, kp, (C2*)b.B, tw, b.err);
             k_zpass<T, NZ, false, false, N><<<zgrid(), thr_zp, sm_zp, s>>>(kp, (C2*)b.B, (const T*)b.chi, (const T*)b.us, b.flag,

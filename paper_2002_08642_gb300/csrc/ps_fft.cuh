@@ -5,8 +5,9 @@
 //
 // Transform convention: X_m = sum_j x_j exp(SIGN * 2 pi i m j / N), no scaling.
 //
-// A length-N line (N = 2^a 3^b) is done in S radix stages: radix 16 while
-// the power-of-two part allows, then its leftover (2, 4 or 8), then radix 3.
+// A length-N line (N = 2^a 3^b) is done in S radix stages: radix RM (16, or 4
+// for short lines) while the power-of-two part allows, then its leftover (2,
+// 4 or 8), then radix 3.
 // Stage s of radix r, with Ls = product of the earlier radices, takes for
 // each butterfly j in [0, N/r) the inputs x[j + t N/r] (t < r), multiplies
 // input t by w^(t k) with k = j mod Ls and w = exp(SIGN 2 pi i / (Ls r)),
@@ -158,33 +159,51 @@ __host__ __device__ constexpr int pow2_part(int n) {
     while (n > 0 && n % 2 == 0) { n /= 2; p *= 2; }
     return p;
 }
-__host__ __device__ constexpr int n_stages(int n) {
+// Largest radix of a line's power-of-two stages. Long lines: 16 (fewest
+// shared-memory round trips). Short lines (n <= 64 and the n = 3M lines over
+// them): 4, so that a line has n / 4 threads instead of n / 16. Radix 4 costs
+// about the same arithmetic per point there (FP64, n = 32: 15 operations
+// against 14), and the passes of small grids are one chain of a few warps per
+// SM.
+// GB300, 32^3 FP64 (this and k_xinv_split): x-forward 52 -> 17 us, z pass
+// 26 -> 14, y passes 12 and 11 -> 8 and 6; 64^3 FP64 x-forward 57 -> 30, z pass
+// 94 -> 70; 48^3 FP32 x-forward 10.4 -> 6.6 (z pass 10.7 -> 11.4).
+#ifndef PS_RADIX4_N
+#define PS_RADIX4_N 64
+#endif
+#ifndef PS_RADIX4_N_F64
+#define PS_RADIX4_N_F64 96
+#endif
+__host__ __device__ constexpr int max_radix(bool fp64, int n) {
+    return n <= (fp64 ? PS_RADIX4_N_F64 : PS_RADIX4_N) ? 4 : 16;
+}
+__host__ __device__ constexpr int n_stages(int n, int rm) {
     int p = pow2_part(n), s = 0;
-    while (p >= 16) { p /= 16; ++s; }
+    while (p >= rm) { p /= rm; ++s; }
     if (p > 1) ++s;
     int q = n / pow2_part(n);
     while (q > 1) { q /= 3; ++s; }
     return s;
 }
-__host__ __device__ constexpr int radix_at(int n, int s) {
+__host__ __device__ constexpr int radix_at(int n, int s, int rm) {
     int p = pow2_part(n), i = 0;
-    while (p >= 16) { if (i == s) return 16; p /= 16; ++i; }
+    while (p >= rm) { if (i == s) return rm; p /= rm; ++i; }
     if (p > 1) { if (i == s) return p; ++i; }
     return 3;
 }
-__host__ __device__ constexpr int ls_at(int n, int s) {
+__host__ __device__ constexpr int ls_at(int n, int s, int rm) {
     int l = 1;
-    for (int i = 0; i < s; ++i) l *= radix_at(n, i);
+    for (int i = 0; i < s; ++i) l *= radix_at(n, i, rm);
     return l;
 }
 // offset of stage s's twiddle block: stages s >= 1 keep (r - 1) Ls entries,
 // entry (t - 1) Ls + k = exp(+2 pi i t k / (Ls r)); the total is n - radix_at(n, 0).
-__host__ __device__ constexpr int tw_offset(int n, int s) {
+__host__ __device__ constexpr int tw_offset(int n, int s, int rm) {
     int o = 0;
-    for (int i = 1; i < s; ++i) o += (radix_at(n, i) - 1) * ls_at(n, i);
+    for (int i = 1; i < s; ++i) o += (radix_at(n, i, rm) - 1) * ls_at(n, i, rm);
     return o;
 }
-__host__ __device__ constexpr int tw_count(int n) { return n - radix_at(n, 0); }
+__host__ __device__ constexpr int tw_count(int n, int rm) { return n - radix_at(n, 0, rm); }
 __host__ __device__ constexpr bool size_ok(int n) {
     int m = n;
     while (m % 2 == 0) m /= 2;
@@ -211,7 +230,9 @@ __device__ __forceinline__ unsigned warp_lanes() {
     return left >= 32 ? 0xffffffffu : ((1u << left) - 1u);
 }
 
-// One length-N line per thread group of G = N / R0 threads. `addr(p)` maps
+// One length-N line per thread group of G = N / R0 threads. RM: largest radix
+// (an n = 3M split's sub-lines take their parent's, so that the thread groups
+// agree). `addr(p)` maps
 // line position p to this thread's shared-memory slot of the tile; `load(p)`
 // feeds the first stage when FROM_TILE is false; `store(p, v)` receives the
 // last stage's outputs (natural order). The caller must __syncthreads()
@@ -219,13 +240,13 @@ __device__ __forceinline__ unsigned warp_lanes() {
 // so every thread of the block must make the call. WS: every line's G
 // threads lie in one warp and touch only their own line's slots, so a warp
 // barrier separates the stages instead of a block barrier.
-template <typename T, int N, int SIGN, bool WS = false> struct LineFFT {
+template <typename T, int N, int SIGN, bool WS = false, int RM = max_radix(sizeof(T) == 8, N)> struct LineFFT {
     using C = cplx<T>;
-    static constexpr int S = n_stages(N);
-    static constexpr int R0 = radix_at(N, 0);
+    static constexpr int S = n_stages(N, RM);
+    static constexpr int R0 = radix_at(N, 0, RM);
     static constexpr int G = N / R0;
     // last stage: radix, butterflies per thread; SLOTS outputs per thread
-    static constexpr int RL = radix_at(N, S - 1);
+    static constexpr int RL = radix_at(N, S - 1, RM);
     static constexpr int NBL = (N / RL + G - 1) / G;
     static constexpr int SLOTS = NBL * RL;
     static_assert(!WS || (G <= 32 && 32 % G == 0), "warp-synchronous lines must not cross warps");
@@ -249,13 +270,13 @@ template <typename T, int N, int SIGN, bool WS = false> struct LineFFT {
     static __device__ __forceinline__ void stage(C* tile, const C* tw, const Addr& addr, int g,
                                                  const Load& load, const Store& store, bool on, unsigned lanes,
                                                  const Hook& hook = Hook()) {
-        constexpr int r = radix_at(N, s);
-        constexpr int Ls = ls_at(N, s);
+        constexpr int r = radix_at(N, s, RM);
+        constexpr int Ls = ls_at(N, s, RM);
         constexpr int NBF = N / r;
         constexpr int NB = (NBF + G - 1) / G;
         constexpr bool last = (s == S - 1);
         constexpr bool from_tile = (s > 0) || FROM_TILE;
-        constexpr int two = tw_offset(N, s);
+        constexpr int two = tw_offset(N, s, RM);
         constexpr bool pad = is_pad16<Addr>::value;
         // one butterfly: inputs, twiddles, DFT
         auto gather = [&](int j, C* v) {

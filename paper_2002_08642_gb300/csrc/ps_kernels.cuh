@@ -190,6 +190,7 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* out, double* 
 // passes' tile widths (at most CW complex, 128-byte rows).
 template <typename T, int N> struct Geo {
     using C2 = cplx<T>;
+    static constexpr int RM = max_radix(sizeof(T) == 8, N);
     static constexpr int G = LineFFT<T, N, 1>::G;
     static constexpr int CW = 128 / (int)sizeof(C2);     // 16 (float), 8 (double)
     static constexpr int LP = N + N / 16;                  // padded z line
@@ -200,7 +201,7 @@ template <typename T, int N> struct Geo {
     // ZNB staging buffers of the batch's six spectral lines plus the FFT tiles
     static constexpr int ZNB = PS_ZP_NBUF == 1 ? 1 : 2;
     static constexpr int zsmem(int l) {
-        return (int)sizeof(C2) * (ZNB * 6 * l * KZP + 3 * l * LP + tw_count(N) + 1) + 128;
+        return (int)sizeof(C2) * (ZNB * 6 * l * KZP + 3 * l * LP + tw_count(N, RM) + 1) + 128;
     }
     // lines of at most 16 threads take batches of 2 lines (measured on GB300:
     // 256^3 z pass 0.187 -> 0.177 ms); longer lines the largest batch within
@@ -234,13 +235,13 @@ template <typename T, int N> struct Geo {
     }
     static constexpr int Y2NB = PS_Y2_NBUF == 1 ? 1 : 2;
     static constexpr int y2_smem(int c, int nb = 2) {   // y inverse: nb staging (K rows) + work tile (N rows)
-        return (int)sizeof(C2) * c * (nb * nbox(K) * bpitch(K, c) + N) + (int)sizeof(C2) * (tw_count(N) + 1) + 256;
+        return (int)sizeof(C2) * c * (nb * nbox(K) * bpitch(K, c) + N) + (int)sizeof(C2) * (tw_count(N, RM) + 1) + 256;
     }
     static constexpr int y4_smem(int c) {   // y forward: 2 staging tiles of N rows, transformed in place
-        return (int)sizeof(C2) * c * (2 * nbox(N) * bpitch(N, c)) + (int)sizeof(C2) * (tw_count(N) + 1) + 256;
+        return (int)sizeof(C2) * c * (2 * nbox(N) * bpitch(N, c)) + (int)sizeof(C2) * (tw_count(N, RM) + 1) + 256;
     }
     static constexpr int x5_smem(int c, int nf = 3) {   // x forward: 2 staging tiles (N rows) + nf result tiles
-        return (int)sizeof(C2) * c * (2 * nbox(N) * bpitch(N, c) + nf * K) + (int)sizeof(C2) * (tw_count(N) + 1) + 256;
+        return (int)sizeof(C2) * c * (2 * nbox(N) * bpitch(N, c) + nf * K) + (int)sizeof(C2) * (tw_count(N, RM) + 1) + 256;
     }
     // widest tile (at most cmax complex, at least 2) whose shared memory fits
     static constexpr int pick_c(int which, int kb, int cmax) {
@@ -258,7 +259,7 @@ template <typename T, int N> struct Geo {
     static constexpr int CY4 = pick_c(4, PS_Y4_SMEM_KB, 16);
     static constexpr int CX1 = pick_c(1, PS_X1_SMEM_KB, 16);   // same smem shape as the y inverse, two buffers
     static constexpr int CX5 = pick_c(5, PS_X5_SMEM_KB, 128 / 16);
-    static constexpr int tw_n = tw_count(N) > 0 ? tw_count(N) : 1;
+    static constexpr int tw_n = tw_count(N, RM) > 0 ? tw_count(N, RM) : 1;
 };
 
 __device__ __forceinline__ int zaddr(int p, int line, int LP) { return line * LP + p + (p >> 4); }
@@ -340,12 +341,15 @@ __device__ __forceinline__ unsigned char* smem_base128(unsigned char* raw) {
 template <typename T, int N> struct Split3 {
     static constexpr bool on = (N % 3 == 0) && (PS_Z3 != 0);
     static constexpr int M = on ? N / 3 : N;
-    static constexpr int GM = LineFFT<T, M, 1>::G;                     // threads per sub-line
-    static constexpr int TWM = on ? (tw_count(M) > 0 ? tw_count(M) : 1) : 0;
+    static constexpr int RM = max_radix(sizeof(T) == 8, N);            // radix of the sub-lines: the line's
+    template <int SIGN, bool WS = false> using FFT = LineFFT<T, M, SIGN, WS, RM>;
+    static constexpr int GM = FFT<1>::G;                               // threads per sub-line
+    static constexpr int TWN = tw_count(M, RM);
+    static constexpr int TWM = on ? (TWN > 0 ? TWN : 1) : 0;
     // the block's thread groups split evenly over the three sub-lines, and
     // the M table plus tw3 fit in the room of the n table (+ 1)
     static_assert(!on || 3 * GM == LineFFT<T, N, 1>::G, "n = 3M split: group count");
-    static_assert(!on || TWM + 2 * M <= tw_count(N) + 1, "n = 3M split: twiddle room");
+    static_assert(!on || TWM + 2 * M <= tw_count(N, RM) + 1, "n = 3M split: twiddle room");
 };
 
 // Z[k] and Z[2M + k] from F_0[k], F_1[k], F_2[k].
@@ -478,7 +482,7 @@ template <typename T, int N>
 __device__ __forceinline__ cplx<T>* load_tw_split(cplx<T>* tw, const cplx<T>* twg, int n_tw) {
     using S3 = Split3<T, N>;
     if constexpr (S3::on) {
-        for (int i = threadIdx.x; i < tw_count(S3::M); i += blockDim.x) tw[i] = twg[N + i];
+        for (int i = threadIdx.x; i < S3::TWN; i += blockDim.x) tw[i] = twg[N + i];
         for (int i = threadIdx.x; i < 2 * S3::M; i += blockDim.x) tw[S3::TWM + i] = twg[2 * N + i];
         return tw + S3::TWM;
     } else {
@@ -535,15 +539,16 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
     using C2 = cplx<T>;
     using GE = Geo<T, N>;
     constexpr int G = GE::G, LZ = GE::LZ, LP = GE::LP, KZP = GE::KZP;
-    constexpr bool Z3 = (N % 3 == 0) && (PS_Z3 != 0);
-    constexpr int M = Z3 ? N / 3 : N;
-    constexpr int GM = LineFFT<T, M, 1>::G;        // threads per sub-line
+    constexpr bool Z3 = Split3<T, N>::on;
+    constexpr int M = Split3<T, N>::M;
+    using S3 = Split3<T, N>;
+    constexpr int GM = S3::GM;        // threads per sub-line
     static_assert(!Z3 || G == 3 * GM, "three sub-lines per line group");
     // a (sub-)line's threads are consecutive and start at a multiple of its
     // thread count: if that count divides 32, its stages need warp barriers only
     constexpr int GL = Z3 ? GM : G;
     constexpr bool WS = PS_ZWS != 0 && GL <= 32 && 32 % GL == 0;
-    constexpr int TWM = Z3 ? (tw_count(M) > 0 ? tw_count(M) : 1) : 0;
+    constexpr int TWM = S3::TWM;
     constexpr int nyl = NY;   // lines per x-plane (= kp.n; the line length is N)
     const int b0 = kp.xs0 * nyl / LZ, b1 = (kp.xs0 + kp.xsn) * nyl / LZ;   // this launch's batches
     constexpr uint32_t fbytes = (uint32_t)(LZ * KZP * sizeof(C2));
@@ -572,7 +577,7 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
     }
     C2* tw3 = tw + TWM;   // n = 3M: e^{+2 pi i b q'/n}, b = 1, 2
     if constexpr (Z3) {
-        if constexpr (tw_count(M) > 0) load_tw(tw, twg + N, tw_count(M));
+        if constexpr (S3::TWN > 0) load_tw(tw, twg + N, S3::TWN);
         load_tw(tw3, twg + 2 * N, 2 * M);
     } else {
         load_tw(tw, twg, GE::tw_n);
@@ -627,11 +632,11 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
             const int tbase = (int)(tile(pl, pr) - tiles);
             auto noload = [&](int) -> C2 { return cmk<C2>((T)0, (T)0); };
             if constexpr (M % 16 == 0) {   // the sub-line starts on a padding group
-                LineFFT<T, M, 1, WS>::template run_tile<true>(tiles, tw, Pad16{tbase + zad(sub * M)}, gm, noload);
+                S3::template FFT<1, WS>::template run_tile<true>(tiles, tw, Pad16{tbase + zad(sub * M)}, gm, noload);
             } else {
                 auto addr = [&](int p) { return tbase + zad(sub * M + p); };
                 auto store = [&](int p, C2 v) { tiles[addr(p)] = v; };
-                LineFFT<T, M, 1, WS>::template run<true>(tiles, tw, addr, gm, noload, store);
+                S3::template FFT<1, WS>::template run<true>(tiles, tw, addr, gm, noload, store);
             }
         } else {
             const C2* fa = st + (size_t)((2 * pr) * LZ + pl) * KZP;
@@ -757,12 +762,12 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
             if constexpr (Z3) {
                 const int sub = g / GM, gm = g % GM;
                 if constexpr (M % 16 == 0) {
-                    LineFFT<T, M, -1, WS>::template run_tile_masked<true>(tiles, tw, Pad16{tbase + zad(sub * M)}, gm,
+                    S3::template FFT<-1, WS>::template run_tile_masked<true>(tiles, tw, Pad16{tbase + zad(sub * M)}, gm,
                                                                           noload, active);
                 } else {
                     auto addr = [&](int p) { return tbase + zad(sub * M + p); };
                     auto store = [&](int p, C2 v) { if (active) tiles[addr(p)] = v; };
-                    LineFFT<T, M, -1, WS>::template run_masked<true>(tiles, tw, addr, gm, noload, store, active);
+                    S3::template FFT<-1, WS>::template run_masked<true>(tiles, tw, addr, gm, noload, store, active);
                 }
             } else {
                 LineFFT<T, N, -1, WS>::template run_tile_masked<true>(tiles, tw, Pad16{tbase}, g, noload, active);
@@ -1015,7 +1020,7 @@ k_yfwd_tma(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict__ 
             const int sub = g / S3::GM, gm = g % S3::GM;
             auto addr3 = [&](int p) { return (int)(Sb - S) + (3 * p + sub) * CT + col; };
             auto store = [&](int p, C2 v) { S[addr3(p)] = v; };
-            LineFFT<T, M, -1>::template run<true>(S, tw, addr3, gm, noload, store);
+            S3::template FFT<-1>::template run<true>(S, tw, addr3, gm, noload, store);
             __syncthreads();
             for (int idx = threadIdx.x; idx < M * CT; idx += blockDim.x) {
                 const int kq = idx / CT, c = idx % CT;
@@ -1165,6 +1170,91 @@ k_xinv_tma(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict__ 
     }
 }
 
+// pass 1 of small grids: the same x-inverse with one item per (ky, kz tile,
+// output field), the vorticity component formed in the first stage's loads
+// from its two velocity fields. Six transforms and nine field loads per tile
+// instead of five and three, but six times the blocks and one transform
+// instead of five in a chain: taken where the tiles do not fill the SMs
+// (Engine::XSPLIT), where the fields sit in L2.
+// GB300: 32^3 FP64 55 -> 7 us, 64^3 FP64 62 -> 23, 48^3 FP32 8.9 -> 4.4 (with the
+// radix 4 of short lines).
+template <typename T, int N, int KZP_ = Geo<T, N>::KZP>
+__global__ void __launch_bounds__(Geo<T, N>::CX1 * Geo<T, N>::G)
+k_xinv_split(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict__ A, const cplx<T>* __restrict__ twg,
+             int* __restrict__ err) {
+    using C2 = cplx<T>;
+    using GE = Geo<T, N>;
+    using FFT = LineFFT<T, N, 1>;
+    constexpr int CT = GE::CX1, K = GE::K;
+    constexpr int NBOX = GE::nbox(K), BR = GE::brows(K), BP = GE::bpitch(K, CT), RS = NBOX * BP;
+    constexpr int KZP = KZP_, NTZ = KZP / CT;
+    const int NITEM = kp.kyn * NTZ * 6;
+    constexpr uint32_t box_bytes = (uint32_t)(BR * CT * sizeof(C2));
+    extern __shared__ __align__(16) unsigned char smraw[];
+    C2* S = reinterpret_cast<C2*>(smem_base128(smraw));   // [2][RS][CT]
+    if (smem_u32(S) & 127u) {
+        if (threadIdx.x == 0) atomicExch(err, 2);
+        return;
+    }
+    C2* W = S + 2 * RS * CT;                              // [N][CT]
+    C2* tw = W + N * CT;
+    __shared__ __align__(8) uint64_t bar;
+    const int col = threadIdx.x % CT, g = threadIdx.x / CT;
+    const int mmax = kp.mmax, Kz = kp.Kz;
+    const size_t AS = (size_t)N * K * KZP;
+    if (threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        fence_mbar_init();
+    }
+    load_tw(tw, twg, GE::tw_n);
+    __syncthreads();
+    auto addr = [&](int p) { return p * CT + col; };
+    int it = 0;
+    for (int i = blockIdx.x; i < NITEM; i += gridDim.x, ++it) {
+        const int f = i % 6, t = i / 6, cy = kp.ky0 + t / NTZ, czt = t % NTZ;
+        // velocity component f, or the two (a, b) of w_c = i (k_a u_b - k_b u_a)
+        const int a = f < 3 ? f : (f + 1) % 3, b = (f + 2) % 3;
+        if (threadIdx.x == 0) {
+            fence_proxy_async();
+            mbar_arrive_expect_tx(&bar, (f < 3 ? 1 : 2) * NBOX * box_bytes);
+            for (int x = 0; x < NBOX; ++x) {
+                tma_load_2d(S + (size_t)(x * BP) * CT, &tm, 2 * czt * CT, (a * K + cy) * K + x * BR, &bar);
+                if (f >= 3)
+                    tma_load_2d(S + (size_t)(RS + x * BP) * CT, &tm, 2 * czt * CT, (b * K + cy) * K + x * BR, &bar);
+            }
+        }
+        const bool ok = mbar_wait(&bar, (uint32_t)(it & 1));
+        if (__syncthreads_or(!ok)) {
+            if (threadIdx.x == 0) {
+                atomicExch(err, 1);
+                mbar_wait(&bar, (uint32_t)(it & 1));
+            }
+            break;
+        }
+        const int cz = czt * CT + col;
+        const bool okz = cz < Kz;
+        const T ks = (T)kp.ks, ky = ks * (T)cmode_of(cy, mmax, K), kz = (T)kp.ksz * (T)cz;
+        auto load = [&](int q) -> C2 {
+            const int m = mode_of(q, N);
+            if (m > mmax || m < -mmax) return cmk<C2>((T)0, (T)0);
+            const int c = cidx_of(m, K);
+            const int o = ((c / BR) * BP + c % BR) * CT + col;
+            const C2 ua = S[o];
+            if (f < 3) return ua;
+            const C2 ub = S[RS * CT + o];
+            const T kx = ks * (T)m;
+            const T ka = a == 0 ? kx : a == 1 ? ky : kz, kb = b == 0 ? kx : b == 1 ? ky : kz;
+            return cmk<C2>(kb * ua.y - ka * ub.y, ka * ub.x - kb * ua.x);
+        };
+        C2* out = A + f * AS + cz;
+        auto store = [&](int x, C2 v) {
+            if (okz) out[GE::arow(x, cy) * KZP] = v;
+        };
+        FFT::template run<false>(W, tw, addr, g, load, store);
+        __syncthreads();
+    }
+}
+
 // pass 5 (TMA-staged): x-forward of the three fields of n, truncation to the
 // kept kx, 1/n^3, Leray projection and the integrating-factor AB2 (Euler on
 // the first step) update of U and H. MODE 1 instead sets U to the projected
@@ -1261,7 +1351,7 @@ k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUten
                 const int sub = g / S3::GM, gm = g % S3::GM;
                 auto addr3 = [&](int p) { return (int)(Sb - S) + (3 * p + sub) * CT + col; };
                 auto store = [&](int p, C2 v) { S[addr3(p)] = v; };
-                LineFFT<T, M, -1>::template run<true>(S, tw, addr3, gm, noload, store);
+                S3::template FFT<-1>::template run<true>(S, tw, addr3, gm, noload, store);
                 __syncthreads();
                 for (int idx = threadIdx.x; idx < M * CT; idx += blockDim.x) {
                     const int kq = idx / CT, c = idx % CT;
