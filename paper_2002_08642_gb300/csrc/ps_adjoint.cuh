@@ -18,19 +18,16 @@
 //   dJ/dus  = (chi/eta) nbar - (dx^3/eta) chi (a + b x r)
 //   lam' += n^3 [forward(ubar) + i k x forward(wbar)]
 #pragma once
+#include "ps_adjoint_z.cuh"
 #include "ps_kernels.cuh"
 
 namespace ps {
 
-struct AdjW {
-    double a[3], b[3];   // dJ/dF, dJ/dM of this step
-    int first;           // reversing the integrating-factor Euler start step
-};
-
-// Spectral part 1: G = P (a1 lam + mu); lam <- E lam; mu <- -0.5 dt E^2 lam.
+// Spectral part: G = P (a1 lam + mu). (The x-forward pass at the end of the
+// reversed step updates lam and mu.)
 template <typename T>
-__global__ void k_adj_spec1(KP kp, cplx<T>* __restrict__ lam, cplx<T>* __restrict__ mu, cplx<T>* __restrict__ G,
-                            const T* __restrict__ Ex, const T* __restrict__ Ez, int first) {
+__global__ void k_adj_spec(KP kp, const cplx<T>* __restrict__ lam, const cplx<T>* __restrict__ mu, cplx<T>* __restrict__ G,
+                           const T* __restrict__ Ex, const T* __restrict__ Ez, int first) {
     using C2 = cplx<T>;
     const int K = kp.K, Kz = kp.Kz, Kzp = kp.Kzp, mm = kp.mmax;
     const size_t FS = (size_t)K * K * Kzp;
@@ -44,12 +41,10 @@ __global__ void k_adj_spec1(KP kp, cplx<T>* __restrict__ lam, cplx<T>* __restric
         const size_t o = ((size_t)cy * K + cx) * Kzp + cz;
         const T E = Ex[cx] * Ex[cy] * Ez[cz];
         const T a1 = first ? dt * E : (T)1.5 * dt * E;
-        const T a2 = first ? (T)0 : (T)0.5 * dt * E * E;
-        C2 g[3], l[3];
+        C2 g[3];
         for (int f = 0; f < 3; ++f) {
-            l[f] = lam[f * FS + o];
-            const C2 m = mu[f * FS + o];
-            g[f] = cmk<C2>(a1 * l[f].x + m.x, a1 * l[f].y + m.y);
+            const C2 l = lam[f * FS + o], m = mu[f * FS + o];
+            g[f] = cmk<C2>(a1 * l.x + m.x, a1 * l.y + m.y);
         }
         const int mx = cmode_of(cx, mm, K), my = cmode_of(cy, mm, K);
         const T kx = s * (T)mx, ky = s * (T)my, kz = sz * (T)cz;
@@ -63,99 +58,7 @@ __global__ void k_adj_spec1(KP kp, cplx<T>* __restrict__ lam, cplx<T>* __restric
             g[1].x -= ky * dr; g[1].y -= ky * di;
             g[2].x -= kz * dr; g[2].y -= kz * di;
         }
-        for (int f = 0; f < 3; ++f) {
-            G[f * FS + o] = g[f];
-            lam[f * FS + o] = cmk<C2>(E * l[f].x, E * l[f].y);
-            mu[f * FS + o] = cmk<C2>(-a2 * l[f].x, -a2 * l[f].y);
-        }
-    }
-}
-
-// lam += n^3 (Ub + i k x Wb).
-template <typename T>
-__global__ void k_adj_spec2(KP kp, cplx<T>* __restrict__ lam, const cplx<T>* __restrict__ Ub,
-                            const cplx<T>* __restrict__ Wb) {
-    using C2 = cplx<T>;
-    const int K = kp.K, Kz = kp.Kz, Kzp = kp.Kzp, mm = kp.mmax;
-    const size_t FS = (size_t)K * K * Kzp;
-    const size_t tot = (size_t)K * K * Kz;
-    const T s = (T)kp.ks, sz = (T)kp.ksz;
-    const T n3 = (T)(1.0 / kp.invn3);
-    // 32-bit index arithmetic: K^2 Kz < 2^27 for every grid the library builds
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < (uint32_t)tot; i += gridDim.x * blockDim.x) {
-        const int cz = (int)(i % (uint32_t)Kz);
-        const uint32_t r = i / (uint32_t)Kz;
-        const int cx = (int)(r % (uint32_t)K), cy = (int)(r / (uint32_t)K);
-        const size_t o = ((size_t)cy * K + cx) * Kzp + cz;
-        const T kx = s * (T)cmode_of(cx, mm, K), ky = s * (T)cmode_of(cy, mm, K), kz = sz * (T)cz;
-        const C2 wx = Wb[o], wy = Wb[FS + o], wz = Wb[2 * FS + o];
-        const C2 c0 = cmk<C2>(ky * wz.x - kz * wy.x, ky * wz.y - kz * wy.y);
-        const C2 c1 = cmk<C2>(kz * wx.x - kx * wz.x, kz * wx.y - kx * wz.y);
-        const C2 c2 = cmk<C2>(kx * wy.x - ky * wx.x, kx * wy.y - ky * wx.y);
-        const C2 cc[3] = {cmk<C2>(-c0.y, c0.x), cmk<C2>(-c1.y, c1.x), cmk<C2>(-c2.y, c2.x)};
-        for (int f = 0; f < 3; ++f) {
-            const C2 u = Ub[f * FS + o];
-            const C2 l = lam[f * FS + o];
-            lam[f * FS + o] = cmk<C2>(l.x + n3 * (u.x + cc[f].x), l.y + n3 * (u.y + cc[f].y));
-        }
-    }
-}
-
-// Physical pointwise adjoint. u, w: velocity and vorticity of the step (3 x
-// n^3 each), overwritten by ubar and wbar; nb: inverse(G) (scaled here by
-// 1/n^3). Writes dJ/dchi and dJ/dus of this step.
-// Memory bound: the thirteen loads of a point are issued before its
-// arithmetic, with a register budget (four blocks of 256 threads per SM) that
-// keeps them all in flight.
-template <typename T>
-__global__ void __launch_bounds__(256, 4) k_adj_point(KP kp, AdjW aw, T* __restrict__ u, T* __restrict__ w, const T* __restrict__ nb,
-                            const T* __restrict__ chi, const T* __restrict__ us, T* __restrict__ gchi,
-                            T* __restrict__ gus) {
-    const int n = kp.n, nz = kp.nz;
-    const size_t n3 = (size_t)n * n * nz;
-    // constants in T: no double arithmetic and no 64-bit division per point
-    const T inv_eta = (T)kp.inv_eta, invn3 = (T)kp.invn3, dx = (T)kp.dx;
-    const T f = (T)(kp.dx * kp.dx * kp.dx * kp.inv_eta);
-    const T x0 = (T)kp.x0[0], y0 = (T)kp.x0[1], z0 = (T)kp.x0[2];
-    const T a0 = (T)aw.a[0], a1 = (T)aw.a[1], a2 = (T)aw.a[2];
-    const T b0 = (T)aw.b[0], b1 = (T)aw.b[1], b2 = (T)aw.b[2];
-    // 32-bit point index (n^3 < 2^32 for every built grid size)
-    const uint32_t n3u = (uint32_t)n3, un = (uint32_t)n, unz = (uint32_t)nz;
-    for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < n3u; p += gridDim.x * blockDim.x) {
-        {
-            const uint32_t q = p / unz, k = p - q * unz;
-            const uint32_t i = q / un, j = q - i * un;
-            const T nbx0 = nb[p], nby0 = nb[n3 + p], nbz0 = nb[2 * n3 + p];
-            const T ux = u[p], uy = u[n3 + p], uz = u[2 * n3 + p];
-            const T wx = w[p], wy = w[n3 + p], wz = w[2 * n3 + p];
-            const T c = chi[p];
-            const T sx = us[p], sy = us[n3 + p], sz = us[2 * n3 + p];
-            const T rx = (T)i * dx - x0, ry = (T)j * dx - y0;
-            const T nbx = nbx0 * invn3, nby = nby0 * invn3, nbz = nbz0 * invn3;
-            const T ce = c * inv_eta;
-            // ubar = w x nbar - c nbar ; wbar = nbar x u
-            T bx = wy * nbz - wz * nby - ce * nbx;
-            T by = wz * nbx - wx * nbz - ce * nby;
-            T bz = wx * nby - wy * nbx - ce * nbz;
-            const T vx = nby * uz - nbz * uy;
-            const T vy = nbz * ux - nbx * uz;
-            const T vz = nbx * uy - nby * ux;
-            // dJ/dchi is needed at every cell (also where chi = 0); the force
-            // and moment term uses dJ/dp = a + b x r, p = chi (u - us)
-            const T dx_ = ux - sx, dy_ = uy - sy, dz_ = uz - sz;
-            const T rz = (T)k * dx - z0;
-            const T gx = a0 + b1 * rz - b2 * ry;
-            const T gy = a1 + b2 * rx - b0 * rz;
-            const T gz = a2 + b0 * ry - b1 * rx;
-            const T cf = f * c;
-            bx += cf * gx; by += cf * gy; bz += cf * gz;
-            const T gc = -inv_eta * (nbx * dx_ + nby * dy_ + nbz * dz_) + f * (gx * dx_ + gy * dy_ + gz * dz_);
-            const T gsx = ce * nbx - cf * gx, gsy = ce * nby - cf * gy, gsz = ce * nbz - cf * gz;
-            u[p] = bx; u[n3 + p] = by; u[2 * n3 + p] = bz;
-            w[p] = vx; w[n3 + p] = vy; w[2 * n3 + p] = vz;
-            gchi[p] = gc;
-            gus[p] = gsx; gus[n3 + p] = gsy; gus[2 * n3 + p] = gsz;
-        }
+        for (int f = 0; f < 3; ++f) G[f * FS + o] = g[f];
     }
 }
 

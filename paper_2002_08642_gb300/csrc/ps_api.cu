@@ -47,9 +47,8 @@ struct ps_ctx {
     CUtensorMap tmP;          // the pressure's Pi_hat in field 3 of A (x-inverse input)
     CUtensorMap tmN;          // keep_uw: the pressure's N fields (y-forward input)
     bool uw_valid;            // keep_uw: B holds u and omega of the current state
-    // adjoint (with_adjoint): lam, mu, G, W, Ub, Wb spectral; u, w, nb physical
-    void* adj_spec[6];
-    void* adj_phys[3];
+    CUtensorMap tmL;          // adjoint lam in x-forward boxes (L2 prefetch)
+    void* adj_spec[3];        // with_adjoint: lam, mu, G (spectral)
     double* gX;               // rasteriser VJP scratch (n_nodes x 3)
     MaskArgs last_mask;       // geometry of the last rasterisation
     bool has_last_mask;
@@ -77,7 +76,7 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 int tile_width(int fp64) { return fp64 ? 8 : 16; }
 
 struct Layout {
-    size_t U, H, A, B, N3, chi, us, flag, tw, Ex, Ez, partial, out, err, mask, adj_spec[6], adj_phys[3], gX, total;
+    size_t U, H, A, B, N3, chi, us, flag, tw, Ex, Ez, partial, out, err, mask, adj_spec[3], NB, gX, total;
     size_t ustate, mask_bytes;
 };
 
@@ -115,9 +114,8 @@ bool layout_for(const ps_params* p, const Ops* ops, Layout* L) {
     L->err = take(256);
     L->mask_bytes = mask_workspace_bytes(n, nz);
     L->mask = take(L->mask_bytes);
-    // lam, mu, G, (unused), Ub, Wb
-    for (int i = 0; i < 6; ++i) L->adj_spec[i] = p->with_adjoint && i != 3 ? take(L->ustate) : 0;
-    for (int i = 0; i < 3; ++i) L->adj_phys[i] = p->with_adjoint ? take(3 * n3 * er) : 0;
+    for (int i = 0; i < 3; ++i) L->adj_spec[i] = p->with_adjoint ? take(L->ustate) : 0;
+    L->NB = p->with_adjoint ? take(3 * (size_t)n * n * Kzp * ec) : 0;
     L->gX = take((size_t)kMaskMaxNodes * 3 * sizeof(double));
     L->total = off;
     return true;
@@ -475,40 +473,17 @@ template cudaError_t ps::rasterise<double>(const MaskArgs&, void*, void*, uint8_
 template <typename T>
 static cudaError_t adjoint_step_t(ps_ctx* c, const AdjW& aw, void* gchi, void* gus) {
     using C2 = cplx<T>;
-    cudaStream_t s = c->stream;
-    // grid-stride passes: exactly the blocks that are resident at once
-    static int spec1_blocks = 0, spec2_blocks = 0, pt_blocks = 0;
-    if (pt_blocks == 0) {
-        int nsm = 0;
+    // grid-stride pass: exactly the blocks that are resident at once
+    static int blocks = 0;
+    if (blocks == 0) {
+        int nsm = 0, occ = 0;
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device);
-        if (nsm < 1) nsm = 1;
-        auto resident = [&](auto kern) {
-            int occ = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 256, 0);
-            return (occ > 0 ? occ : 1) * nsm;
-        };
-        spec1_blocks = resident(k_adj_spec1<T>);
-        spec2_blocks = resident(k_adj_spec2<T>);
-        pt_blocks = resident(k_adj_point<T>);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_adj_spec<T>, 256, 0);
+        blocks = (occ > 0 ? occ : 1) * (nsm > 0 ? nsm : 1);
     }
-    C2* lam = (C2*)c->adj_spec[0];
-    C2* mu = (C2*)c->adj_spec[1];
-    C2* G = (C2*)c->adj_spec[2];
-    C2* Ub = (C2*)c->adj_spec[4];
-    C2* Wb = (C2*)c->adj_spec[5];
-    T* up = (T*)c->adj_phys[0];
-    T* wp = (T*)c->adj_phys[1];
-    T* np_ = (T*)c->adj_phys[2];
-    cudaError_t e;
-    k_adj_spec1<T><<<spec1_blocks, 256, 0, s>>>(c->kp, lam, mu, G, (const T*)c->b.Ex, (const T*)c->b.Ez, aw.first);
-    if ((e = c->ops->inv_uw(c->kp, c->b, up, wp, s)) != cudaSuccess) return e;
-    if ((e = c->ops->inv_g(c->kp, c->b, np_, s)) != cudaSuccess) return e;
-    k_adj_point<T><<<pt_blocks, 256, 0, s>>>(c->kp, aw, up, wp, np_, (const T*)c->b.chi, (const T*)c->b.us, (T*)gchi,
-                                          (T*)gus);
-    if ((e = c->ops->fwd3(c->kp, c->b, up, Ub, s)) != cudaSuccess) return e;
-    if ((e = c->ops->fwd3(c->kp, c->b, wp, Wb, s)) != cudaSuccess) return e;
-    k_adj_spec2<T><<<spec2_blocks, 256, 0, s>>>(c->kp, lam, Ub, Wb);
-    return cudaGetLastError();
+    k_adj_spec<T><<<blocks, 256, 0, c->stream>>>(c->kp, (const C2*)c->adj_spec[0], (const C2*)c->adj_spec[1],
+                                                 (C2*)c->adj_spec[2], (const T*)c->b.Ex, (const T*)c->b.Ez, aw.first);
+    return c->ops->adjoint(c->kp, c->b, aw, c->adj_spec[0], c->adj_spec[1], gchi, gus, c->stream);
 }
 
 extern "C" {
@@ -607,8 +582,8 @@ ps_status ps_init(const ps_params* p, void* cuda_stream, void* workspace_dev, si
     c->out = (double*)(w + L.out);
     c->b.err = (int*)(w + L.err);
     c->mask_ws = w + L.mask;
-    for (int i = 0; i < 6; ++i) c->adj_spec[i] = p->with_adjoint && i != 3 ? (void*)(w + L.adj_spec[i]) : nullptr;
-    for (int i = 0; i < 3; ++i) c->adj_phys[i] = p->with_adjoint ? (void*)(w + L.adj_phys[i]) : nullptr;
+    for (int i = 0; i < 3; ++i) c->adj_spec[i] = p->with_adjoint ? (void*)(w + L.adj_spec[i]) : nullptr;
+    c->b.NB = p->with_adjoint ? (void*)(w + L.NB) : nullptr;
     c->gX = (double*)(w + L.gX);
     c->mask_ws_bytes = L.mask_bytes;
 
@@ -642,13 +617,16 @@ ps_status ps_init(const ps_params* p, void* cuda_stream, void* workspace_dev, si
         c->b.tmUp = &c->tmUp;
         c->b.tmHp = &c->tmHp;
         c->b.tmG = nullptr;
+        c->b.tmL = nullptr;
         c->b.chi_sp = nullptr;
         if (p->with_adjoint) {
-            if (!encode_rows(&c->tmG, c->adj_spec[2], c->fp64, (size_t)3 * Kk * Kk, kp.Kzp, ops->cx1, ops->br2)) {
+            if (!encode_rows(&c->tmG, c->adj_spec[2], c->fp64, (size_t)3 * Kk * Kk, kp.Kzp, ops->cx1, ops->br2) ||
+                !encode_rows(&c->tmL, c->adj_spec[0], c->fp64, (size_t)3 * Kk * Kk, kp.Kzp, ops->cx5, ops->br2)) {
                 delete c;
                 return PS_ECUDA;
             }
             c->b.tmG = &c->tmG;
+            c->b.tmL = &c->tmL;
         }
         if (p->keep_uw) {
             if (!encode_rows(&c->tmN, c->b.N3, c->fp64, (size_t)3 * n * n, kp.Kzp, ops->cy4, ops->br4)) {

@@ -3,6 +3,7 @@
 // function pointers so that the C ABI can dispatch on the runtime grid size.
 #pragma once
 #include "ps_kernels.cuh"
+#include "ps_adjoint_z.cuh"
 
 // x-inverse: at most this many (ky, kz tile) tiles take the split kernel
 #ifndef PS_XSPLIT_TILES
@@ -33,6 +34,8 @@ struct Bufs {
     const CUtensorMap* tmHp;
     const CUtensorMap* tmG;  // adjoint G as rows of 2 Kzp reals, x-inverse box (null without adjoint)
     const void* chi_sp;      // sponge mask (n^3, caller-owned), null when the sponge term is off
+    const CUtensorMap* tmL;  // adjoint lam as rows of 2 Kzp reals, x-forward box (L2 prefetch)
+    void* NB;                // adjoint: 3 z-spectral fields of nbar [f][x][y][kz] (else null)
     void* N3;                // keep_uw: 3 z-spectral fields [f][x][y][kz] for the pressure's N (else null)
     const CUtensorMap* tmN;  // N3 as rows of 2 Kzp reals (y-forward input), keep_uw only
 };
@@ -50,13 +53,9 @@ struct Ops {
     cudaError_t (*step)(const KP&, const Bufs&, int first, int resume, cudaStream_t, cudaEvent_t* ev);
     cudaError_t (*set_velocity)(const KP&, const Bufs&, const void* u, cudaStream_t);
     cudaError_t (*get_velocity)(const KP&, const Bufs&, void* u, cudaStream_t);
-    // forward transform of 3 physical fields (3 x n^2 nz) to a compact spectral
-    // array (3 x [ky][kx][kz]); A, B are used as scratch
-    cudaError_t (*fwd3)(const KP&, const Bufs&, const void* phys, void* spec, cudaStream_t);
-    // physical u and omega of the state in U (A, B used as scratch)
-    cudaError_t (*inv_uw)(const KP&, const Bufs&, void* u, void* w, cudaStream_t);
-    // physical inverse of the adjoint array G (needs b.tmG)
-    cudaError_t (*inv_g)(const KP&, const Bufs&, void* phys, cudaStream_t);
+    // one reversed step on the adjoint state lam, mu; G holds P(a1 lam + mu)
+    // (needs b.tmG, b.tmL, b.NB; A, B used as scratch)
+    cudaError_t (*adjoint)(const KP&, const Bufs&, const AdjW&, void* lam, void* mu, void* gchi, void* gus, cudaStream_t);
     // static pressure of the state in U with the current mask (n^3 real)
     cudaError_t (*pressure)(const KP&, const Bufs&, void* p, int resume, cudaStream_t);
     // one phase of the step on a slab (kp.xs0/xsn x-planes, kp.ky0/kyn ky
@@ -121,6 +120,15 @@ template <typename T, int N, int NZ = N> struct Engine {
         return g;
     }
     static int& x1grid() {
+        static int g = 0;
+        return g;
+    }
+    using AZ = AdjZ<T, NZ>;
+    static int& zagrid() {   // persistent blocks of the adjoint z pass
+        static int g = 0;
+        return g;
+    }
+    static int& x5agrid() {
         static int g = 0;
         return g;
     }
@@ -197,7 +205,15 @@ template <typename T, int N, int NZ = N> struct Engine {
         if ((e = attr(k_xfwd_tma<T, N, 0, false, KZ_>, sm_x5t))) return e;
         if ((e = attr(k_xfwd_tma<T, N, 1, false, KZ_>, sm_x5t))) return e;
         if ((e = attr(k_xfwd_tma<T, N, 2, false, KZ_>, sm_x5t))) return e;
-        if ((e = attr(k_xfwd_tma<T, N, 3, false, KZ_>, sm_x5t))) return e;
+        if ((e = attr(k_xfwd_tma<T, N, 3, true, KZ_>, sm_x5s))) return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xfwd_tma<T, N, 3, true, KZ_>, thr_x5, sm_x5s)))
+            return e;
+        x5agrid() = nsm * (occ < 1 ? 1 : occ);
+        if ((e = attr(k_adj_zpass<T, NZ, N>, AZ::smem))) return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_adj_zpass<T, NZ, N>, AZ::threads, AZ::smem)))
+            return e;
+        const int nab = N * N / 2;
+        zagrid() = nsm * (occ < 1 ? 1 : occ) < nab ? nsm * (occ < 1 ? 1 : occ) : nab;
         if ((e = attr(k_xfwd_tma<T, N, 0, true, KZ_>, sm_x5s))) return e;
         if ((e = attr(k_zpass<T, NZ, false, true, N>, sm_zp))) return e;
         if ((e = attr(k_yfwd_tma<T, N, GE::CY4, 6, KZ_>, sm_y4))) return e;
@@ -267,34 +283,37 @@ template <typename T, int N, int NZ = N> struct Engine {
         return cudaGetLastError();
     }
 
-    // physical (3 x n^2 nz) inverse transform of the three spectral fields
-    // that tm maps (U, or the adjoint array G)
-    static cudaError_t inverse3(const KP& kp, const Bufs& b, const CUtensorMap& tm, void* phys, cudaStream_t s) {
-        const C2* tw = (const C2*)b.tw;
-        KP k1 = kp;
-        k1.xs0 = 0; k1.xsn = N; k1.part_off = 0;
-        k_xinv_tma<T, N, 3, KZ_><<<x1pgrid(), thr_x1, sm_x1, s>>>(tm, k1, (C2*)b.A, tw, b.err);
-        k_yinv_tma<T, N, 3, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, (C2*)b.B, tw, b.err);
-        k_zinv_phys<T, NZ><<<zigrid(), thr_zi, sm_zi, s>>>(k1, (const C2*)b.B, (T*)phys, twz(b.tw), b.err);
-        return cudaGetLastError();
-    }
     static cudaError_t get_velocity(const KP& kp, const Bufs& b, void* u, cudaStream_t s) {
-        return inverse3(kp, b, *b.tmU, u, s);
-    }
-
-    static cudaError_t fwd3(const KP& kp, const Bufs& b, const void* phys, void* spec, cudaStream_t s) {
         const C2* tw = (const C2*)b.tw;
         KP k1 = kp;
         k1.xs0 = 0; k1.xsn = N; k1.part_off = 0;
-        k_zfwd_phys<T, NZ><<<zfgrid(), thr_zf, sm_zf, s>>>(k1, (const T*)phys, (C2*)b.B, twz(b.tw), b.err);
-        k_yfwd_tma<T, N, GE::CY4, 3, KZ_><<<y4grid(), thr_y4, sm_y4, s>>>(*b.tmB, k1, (C2*)b.A, tw, b.err);
-        k_xfwd_tma<T, N, 2, false, KZ_><<<x5grid(), thr_x5, sm_x5t, s>>>(*b.tmA5, *b.tmUp, *b.tmHp, k1, (C2*)spec, nullptr,
-                                                            (const T*)b.Ex, (const T*)b.Ez, 0, tw, b.err);
+        k_xinv_tma<T, N, 3, KZ_><<<x1pgrid(), thr_x1, sm_x1, s>>>(*b.tmU, k1, (C2*)b.A, tw, b.err);
+        k_yinv_tma<T, N, 3, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, (C2*)b.B, tw, b.err);
+        k_zinv_phys<T, NZ><<<zigrid(), thr_zi, sm_zi, s>>>(k1, (const C2*)b.B, (T*)u, twz(b.tw), b.err);
         return cudaGetLastError();
     }
 
-    static cudaError_t inv_g(const KP& kp, const Bufs& b, void* phys, cudaStream_t s) {
-        return inverse3(kp, b, *b.tmG, phys, s);
+    // reversed step: u and omega of the state U through the step's x (curl
+    // fused) and y passes, nbar = inverse(G) through their plain variants,
+    // the z pass with the pointwise adjoint, the y-forward pass of its six
+    // fields, and the x-forward pass with the update of lam and mu
+    static cudaError_t adjoint(const KP& kp, const Bufs& b, const AdjW& aw, void* lam, void* mu, void* gchi, void* gus,
+                               cudaStream_t s) {
+        const C2* tw = (const C2*)b.tw;
+        KP k1 = kp;
+        k1.xs0 = 0; k1.xsn = N; k1.part_off = 0;
+        k_xinv_tma<T, N, 3, KZ_><<<x1pgrid(), thr_x1, sm_x1, s>>>(*b.tmG, k1, (C2*)b.A, tw, b.err);
+        k_yinv_tma<T, N, 3, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, (C2*)b.NB, tw, b.err);
+        x_inverse(k1, b, s);
+        k_yinv_tma<T, N, 6, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, (C2*)b.B, tw, b.err);
+        k_adj_zpass<T, NZ, N><<<zagrid(), AZ::threads, AZ::smem, s>>>(k1, aw, (C2*)b.B, (const C2*)b.NB, (const T*)b.chi,
+                                                                     (const T*)b.us, b.flag, (T*)gchi, (T*)gus,
+                                                                     twz(b.tw), b.err);
+        k_yfwd_tma<T, N, GE::CY4, 6, KZ_><<<y4grid(), thr_y4, sm_y4, s>>>(*b.tmB, k1, (C2*)b.A, tw, b.err);
+        k_xfwd_tma<T, N, 3, true, KZ_><<<x5agrid(), thr_x5, sm_x5s, s>>>(*b.tmA5, *b.tmL, *b.tmL, k1, (C2*)lam, (C2*)mu,
+                                                                       (const T*)b.Ex, (const T*)b.Ez, aw.first, tw,
+                                                                       b.err);
+        return cudaGetLastError();
     }
 
     // static pressure p = Pi - (1/2)|u|^2 of the state U with the current
@@ -320,25 +339,11 @@ template <typename T, int N, int NZ = N> struct Engine {
         k_yfwd_tma<T, N, GE::CY4, 3, KZ_><<<y4grid(), thr_y4, sm_y4, s>>>(b.N3 ? *b.tmN : *b.tmB, k1, (C2*)b.A, tw,
                                                                   b.err);
         C2* pih = (C2*)b.A + (size_t)3 * N * GE::K * kp.Kzp;
-        k_xfwd_tma<T, N, 3, false, KZ_><<<x5grid(), thr_x5, sm_x5t, s>>>(*b.tmA5, *b.tmUp, *b.tmHp, k1, pih, nullptr,
+        k_xfwd_tma<T, N, 2, false, KZ_><<<x5grid(), thr_x5, sm_x5t, s>>>(*b.tmA5, *b.tmUp, *b.tmHp, k1, pih, nullptr,
                                                             (const T*)b.Ex, (const T*)b.Ez, 0, tw, b.err);
         k_xinv_tma<T, N, 1, KZ_><<<x1pgrid(), thr_x1, sm_x1, s>>>(*b.tmP, k1, (C2*)b.A, tw, b.err);
         k_yinv_tma<T, N, 1, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, nout, tw, b.err);
         k_zinv_sub<T, NZ><<<zsgrid(), thr_zs, sm_zs, s>>>(k1, (const C2*)nout, (T*)p, twz(b.tw), b.err);
-        return cudaGetLastError();
-    }
-
-    // u and omega = curl u of the state U, physical (3 x n^3 each): the
-    // step's x (curl fused) and y passes, then z c2r of fields 0..2 and 3..5
-    static cudaError_t inv_uw(const KP& kp, const Bufs& b, void* u, void* w, cudaStream_t s) {
-        const C2* tw = (const C2*)b.tw;
-        KP k1 = kp;
-        k1.xs0 = 0; k1.xsn = N; k1.part_off = 0;
-        x_inverse(k1, b, s);
-        k_yinv_tma<T, N, 6, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, (C2*)b.B, tw, b.err);
-        const size_t BS = (size_t)N * N * k1.Kzp;
-        k_zinv_phys<T, NZ><<<zigrid(), thr_zi, sm_zi, s>>>(k1, (const C2*)b.B, (T*)u, twz(b.tw), b.err);
-        k_zinv_phys<T, NZ><<<zigrid(), thr_zi, sm_zi, s>>>(k1, (const C2*)b.B + 3 * BS, (T*)w, twz(b.tw), b.err);
         return cudaGetLastError();
     }
 
@@ -369,9 +374,7 @@ template <typename T, int N, int NZ = N> struct Engine {
         o.step = &step;
         o.set_velocity = &set_velocity;
         o.get_velocity = &get_velocity;
-        o.fwd3 = &fwd3;
-        o.inv_uw = &inv_uw;
-        o.inv_g = &inv_g;
+        o.adjoint = &adjoint;
         o.pressure = &pressure;
         o.slab_phase = &slab_phase;
         o.zalign = GZ::LZ;

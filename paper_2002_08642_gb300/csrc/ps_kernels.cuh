@@ -378,18 +378,19 @@ __device__ __forceinline__ void split3_out(C2 F0, C2 F1, C2 F2, const C2* tw3, i
 // round-off of real fields, dropped) and the self-mirror mode M/2.
 // Padded tile position of entry p of sub-line b (sub-lines of length M):
 // zaddr(b M + p) = b (M + M/16) + zaddr(p) when 16 divides M.
-template <int M>
+// (SUB > 0: a sub-line stride other than that).
+template <int M, int SUB = 0>
 __device__ __forceinline__ int zsub(int b, int p) {
-    if constexpr (M % 16 == 0) return b * (M + M / 16) + p + (p >> 4);
+    if constexpr (M % 16 == 0) return b * (SUB > 0 ? SUB : M + M / 16) + p + (p >> 4);
     else return zaddr(b * M + p, 0, 0);
 }
 
-template <typename T, int M>
+template <typename T, int M, int SUB = 0>
 __device__ __forceinline__ void split3_pre(const cplx<T>* fa, const cplx<T>* fb, const cplx<T>* tw3, cplx<T>* t,
                                            int q) {
     using C2 = cplx<T>;
     const T h = (T)0.86602540378443864676;   // sin(2 pi / 3)
-    auto put = [&](int b, int p, C2 v) { t[zsub<M>(b, p)] = v; };
+    auto put = [&](int b, int p, C2 v) { t[zsub<M, SUB>(b, p)] = v; };
     // x + e^{2 pi i 2/3} y, x + e^{-2 pi i 2/3} y  (e^{+-2 pi i 2/3} = (-1/2, -+h))
     auto rm = [&](C2 x, C2 y) { return cmk<C2>(x.x - (T)0.5 * y.x + h * y.y, x.y - (T)0.5 * y.y - h * y.x); };
     auto rp = [&](C2 x, C2 y) { return cmk<C2>(x.x - (T)0.5 * y.x - h * y.y, x.y - (T)0.5 * y.y + h * y.x); };
@@ -429,12 +430,12 @@ __device__ __forceinline__ void split3_pre(const cplx<T>* fa, const cplx<T>* fb,
 //   Z[n - k] = F_0[m] + H_1 + H_2,  Z[m] = F_0[m] + w^2 H_1 + w H_2.
 // k = 0 gives Z[0] (twice) and the self-mirror mode M/2: zm = Z[M/2],
 // znm = Z[n - M/2].
-template <typename T, int M>
+template <typename T, int M, int SUB = 0>
 __device__ __forceinline__ void split3_pair_out(const cplx<T>* t, const cplx<T>* tw3, int k, cplx<T>& zk,
                                                 cplx<T>& znk, cplx<T>& zm, cplx<T>& znm) {
     using C2 = cplx<T>;
     const T h = (T)0.86602540378443864676;
-    auto at = [&](int b, int p) { return t[zsub<M>(b, p)]; };
+    auto at = [&](int b, int p) { return t[zsub<M, SUB>(b, p)]; };
     // x + w y + w^2 z
     auto rw = [&](C2 x, C2 y, C2 z) {
         return cmk<C2>(x.x - (T)0.5 * (y.x + z.x) - h * (y.y - z.y), x.y - (T)0.5 * (y.y + z.y) + h * (y.x - z.x));
@@ -1258,11 +1259,13 @@ k_xinv_split(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict_
 // pass 5 (TMA-staged): x-forward of the three fields of n, truncation to the
 // kept kx, 1/n^3, Leray projection and the integrating-factor AB2 (Euler on
 // the first step) update of U and H. MODE 1 instead sets U to the projected
-// field (mean kept) and clears H; MODE 2 writes the truncated transform
-// times 1/n^3 to U (no projection; H unused); MODE 3 writes the total
+// field (mean kept) and clears H; MODE 2 writes the total
 // pressure coefficients Pi_hat = -i (k . N_hat) / |k|^2 (one field) to U,
-// the gradient part the projection removes. Each field is transformed in
-// place in its staging buffer; kept outputs go to three result tiles.
+// the gradient part the projection removes. MODE 3 (with the six fields of
+// SP) updates the adjoint state U = lam, H = mu: lam <- E lam + (transform of
+// fields 0..2) + i k x (transform of fields 3..5), unscaled, and
+// mu <- -(dt/2) E^2 lam (0 for the Euler start step). Each field is
+// transformed in place in its staging buffer; kept outputs go to three result tiles.
 // tm: A as rows of 2 Kzp reals, row (f K + ky) n + x.
 template <typename T, int N, int MODE, bool SP = false, int KZP_ = Geo<T, N>::KZP>
 __global__ void __launch_bounds__(Geo<T, N>::CX5 * Geo<T, N>::G)
@@ -1323,9 +1326,9 @@ k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUten
         // U (first step) or Q of this tile is read only after the three
         // transforms: start pulling it into L2 now (measured: loading it into
         // registers here instead, held across the transforms, was slower)
-        if (MODE == 0 && threadIdx.x < 3 * NBK) {
+        if ((MODE == 0 || MODE == 3) && threadIdx.x < 3 * NBK) {
             const int f = threadIdx.x / NBK, b = threadIdx.x % NBK;
-            tma_prefetch_2d(first ? &tmu : &tmh, 2 * czt * CT, (f * K + cy) * K + b * BRK);
+            tma_prefetch_2d(MODE == 3 || first ? &tmu : &tmh, 2 * czt * CT, (f * K + cy) * K + b * BRK);
         }
 #pragma unroll 1
         for (int j = 0; j < NF; ++j) {
@@ -1378,7 +1381,7 @@ k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUten
             }
             __syncthreads();
             if constexpr (SP) {
-                if (j == 2) {   // s_hat complete: replace it by the sponge term
+                if (j == 2) {   // s_hat complete: replace it by the sponge term (MODE 3: by i k x s_hat)
                     const T myy = (T)cmode_of(cy, mmax, K);
                     for (int idx = threadIdx.x; idx < K * CT; idx += blockDim.x) {
                         const int cx = idx / CT, czz = czt * CT + idx % CT;
@@ -1387,7 +1390,7 @@ k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUten
                         const T k2 = kx * kx + ky * ky + kz * kz;
                         const C2 s0 = Rt[idx], s1 = Rt[K * CT + idx], s2 = Rt[2 * K * CT + idx];
                         const bool zero = (mx == 0 && cy == 0 && czz == 0);
-                        const T fsp = zero ? (T)0 : -(T)kp.inv_csp / k2;
+                        const T fsp = MODE == 3 ? (T)1 : zero ? (T)0 : -(T)kp.inv_csp / k2;
                         // i (k x s): (re, im) -> (-im, re)
                         const T ax = ky * s2.x - kz * s1.x, bx = ky * s2.y - kz * s1.y;
                         const T ay = kz * s0.x - kx * s2.x, by = kz * s0.y - kx * s2.y;
@@ -1438,15 +1441,21 @@ k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUten
 #pragma unroll
                 for (int ff = 0; ff < 3; ++ff) uq[ff] = first ? U[ff * FS + o] : H[ff * FS + o];
             }
-            if constexpr (MODE == 2) {
+            if constexpr (MODE == 3) {
+                C2 l[3];
+#pragma unroll
+                for (int ff = 0; ff < 3; ++ff) l[ff] = U[ff * FS + o];
+                const T E = Ex[cx] * ey * Ez[czz];
+                const T a2 = first ? (T)0 : (T)0.5 * dt * E * E;
 #pragma unroll
                 for (int ff = 0; ff < 3; ++ff) {
                     const C2 v = Rt[ff * K * CT + idx];
-                    U[ff * FS + o] = cmk<C2>(v.x * invn3, v.y * invn3);
+                    U[ff * FS + o] = cmk<C2>(E * l[ff].x + v.x, E * l[ff].y + v.y);
+                    H[ff * FS + o] = cmk<C2>(-a2 * l[ff].x, -a2 * l[ff].y);
                 }
                 continue;
             }
-            if constexpr (MODE == 3) {   // Pi_hat = -i (k . N_hat) / |k|^2, Pi_hat(0) = 0
+            if constexpr (MODE == 2) {   // Pi_hat = -i (k . N_hat) / |k|^2, Pi_hat(0) = 0
                 const int mx = cmode_of(cx, mmax, K);
                 const T kx = s * (T)mx, ky = s * my, kz = sz * (T)czz;
                 const T k2 = kx * kx + ky * ky + kz * kz;

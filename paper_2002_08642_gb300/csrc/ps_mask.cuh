@@ -41,7 +41,10 @@
 // bound of the distance leaves, 32 at a time.
 // GB300, each kernel alone on the device, against clear + boxes + prefix sum +
 // pair pass(es) + evaluate: 121 nodes at 48^3 FP32 48 -> 28 us (6 + 5 + 17),
-// 600 nodes at 128^3 FP64 229 -> 107 us (8 + 24 + 29 + 29 + 17).
+// 600 nodes at 128^3 FP64 229 -> 107 us (8 + 24 + 29 + 29 + 17). Then sign tests
+// and bound conversions on the integer pipe, the cosine as a series on its half
+// period and node velocities rotated once: wing 48^3 663 -> 632 us (8 steps),
+// 128^3 FP64 3000 -> 2896 (2 steps), FP64 gradient window 64^3 8.9 -> 8.4 ms.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
