@@ -78,7 +78,7 @@ enum { PS_MEAN_FIXED = 0, PS_MEAN_FREE = 1 };
  *   mean_mode  PS_MEAN_FIXED: the k = 0 mode of the right-hand side is
  *              dropped (mean velocity fixed); PS_MEAN_FREE: kept.
  *   with_adjoint  1: the workspace also holds the adjoint state and scratch
- *              (six spectral state arrays and nine physical fields more).
+ *              (three spectral state arrays and three z-spectral fields more).
  *   L, nu, eta, dt  box length, kinematic viscosity, penalization constant,
  *              time step (all > 0).
  *   tw, h      wing semi-thickness and smoothing semi-width of the mask.

@@ -28,6 +28,7 @@ namespace ps {
 template <typename T>
 __global__ void k_adj_spec(KP kp, const cplx<T>* __restrict__ lam, const cplx<T>* __restrict__ mu, cplx<T>* __restrict__ G,
                            const T* __restrict__ Ex, const T* __restrict__ Ez, int first) {
+    pdl_wait();
     using C2 = cplx<T>;
     const int K = kp.K, Kz = kp.Kz, Kzp = kp.Kzp, mm = kp.mmax;
     const size_t FS = (size_t)K * K * Kzp;
@@ -167,6 +168,7 @@ __device__ void vjp_point(const MaskWs& m, const MaskArgs& a, uint32_t p, int t,
 template <typename T>
 __global__ void k_mask_vjp_list(MaskWs m, MaskArgs a, int par, const T* __restrict__ gchi,
                                 const T* __restrict__ gus, const T* __restrict__ chi, double* __restrict__ gX) {
+    pdl_wait();
     const unsigned long long cnt = m.cnt[par];
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
          i += (unsigned long long)gridDim.x * blockDim.x) {
@@ -180,6 +182,7 @@ __global__ void k_mask_vjp_list(MaskWs m, MaskArgs a, int par, const T* __restri
 template <typename T>
 __global__ void k_mask_vjp_dense(MaskWs m, MaskArgs a, const T* __restrict__ gchi, const T* __restrict__ gus,
                                  const T* __restrict__ chi, double* __restrict__ gX) {
+    pdl_wait();
     const size_t n = a.n, nz = a.nz, n3 = n * n * nz;
     for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < n3; p += (size_t)gridDim.x * blockDim.x) {
         const int k = (int)(p % nz), j = (int)((p / nz) % n), i = (int)(p / (n * nz));
@@ -203,6 +206,7 @@ __global__ void k_mask_vjp_dense(MaskWs m, MaskArgs a, const T* __restrict__ gch
 
 // grad_xw[v] += R^T gX[v]  (global -> wing frame)
 __global__ void k_vjp_to_wing(MaskArgs a, const double* __restrict__ gX, double* __restrict__ gxw) {
+    pdl_wait();
     const int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= a.n_nodes) return;
     for (int c = 0; c < 3; ++c) {

@@ -63,6 +63,7 @@ k_adj_zpass(KP kp, AdjW aw, cplx<T>* __restrict__ B, const cplx<T>* __restrict__
     extern __shared__ __align__(16) unsigned char smraw[];
     C2* stage = reinterpret_cast<C2*>(smem_base128(smraw));   // [9][2][KZP]
     if (smem_u32(stage) & 127u) {   // never expected: refuse to start copies
+        pdl_wait();
         if (threadIdx.x == 0) atomicExch(err, 2);
         return;
     }
@@ -80,6 +81,7 @@ k_adj_zpass(KP kp, AdjW aw, cplx<T>* __restrict__ B, const cplx<T>* __restrict__
     }
     C2* tw3 = load_tw_split<T, N>(tw, twg, GE::tw_n);
     __syncthreads();
+    pdl_wait();
     auto issue = [&](int b) {  // one thread
         fence_proxy_async();
         mbar_arrive_expect_tx(&bar, 9 * fbytes);

@@ -275,6 +275,7 @@ void host_tables(const ps_params* p, std::vector<unsigned char>& tw, std::vector
 // ------------------------------------------------------ generic kernels
 template <typename T>
 __global__ void k_line_flags(const T* __restrict__ chi, uint8_t* __restrict__ flag, int n, int nz) {
+    pdl_wait();
     const long line = (long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     const int lane = threadIdx.x & 31;
     if (line >= (long)n * n) return;
@@ -298,6 +299,7 @@ static constexpr int kForceThreads = 128;
 __global__ void __launch_bounds__(kForceThreads)
 k_force_final(const double* __restrict__ part, int nb, double scale, const int* __restrict__ err,
               double* __restrict__ out) {
+    pdl_wait();
     __shared__ Acc sh[kForceThreads / 32];
     const int i = blockIdx.x;
     Acc a = {0, 0};
@@ -323,6 +325,7 @@ k_force_final(const double* __restrict__ part, int nb, double scale, const int* 
 // Energy, max |k . c| and a non-finite count over the spectral state.
 template <typename T>
 __global__ void k_diag(KP kp, const cplx<T>* __restrict__ U, double* __restrict__ part) {
+    pdl_wait();
     __shared__ double red[32 * 3];
     const int K = kp.K, Kz = kp.Kz, Kzp = kp.Kzp, mm = kp.mmax;
     const size_t FS = (size_t)K * K * Kzp;
@@ -368,6 +371,7 @@ __global__ void k_diag(KP kp, const cplx<T>* __restrict__ U, double* __restrict_
 // caller-chosen cap; on giving up the block records the device error flag
 // the way the transform passes do. Nothing is in flight when it returns.
 __global__ void k_wait_timeout(int* __restrict__ err, uint32_t cap) {
+    pdl_wait();
     __shared__ __align__(8) uint64_t bar;
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
@@ -381,6 +385,7 @@ __global__ void k_wait_timeout(int* __restrict__ err, uint32_t cap) {
 }
 
 __global__ void k_diag_final(const double* __restrict__ part, int nb, double half_L3, double* __restrict__ out) {
+    pdl_wait();
     if (threadIdx.x != 0) return;
     Acc e = {0, 0};
     double m = 0.0, bad = 0.0;
@@ -440,12 +445,12 @@ cudaError_t ps::rasterise(const MaskArgs& a, void* chi, void* us, uint8_t* flag,
     const int most = std::max(std::max(a.n_nodes, 4 * a.n_tri), 256 * 4 * kRasterSM);
     const int cb = (most + 255) / 256;
     if (a.profile == PS_MASK_TANH) {
-        k_mask_prepare<T, false><<<cb, 256, 0, s>>>(m, a, par, (T*)chi, (T*)us, flag, n3, n * n, 0.0);
-        k_mask_dense<T><<<16 * kRasterSM, 128, 0, s>>>(m, a, (T*)chi, (T*)us, flag);
+        launch(k_mask_prepare<T, false>, cb, 256, 0, s, m, a, par, (T*)chi, (T*)us, flag, n3, n * n, 0.0);
+        launch(k_mask_dense<T>, 16 * kRasterSM, 128, 0, s, m, a, (T*)chi, (T*)us, flag);
         *par_out = np;  // both lists empty: the next call must clear densely
         return cudaGetLastError();
     }
-    k_mask_prepare<T, true><<<cb, 256, 0, s>>>(m, a, par, (T*)chi, (T*)us, flag, n3, n * n, a.tw + a.h);
+    launch(k_mask_prepare<T, true>, cb, 256, 0, s, m, a, par, (T*)chi, (T*)us, flag, n3, n * n, a.tw + a.h);
     // FP32: about 32 warps per SM over the triangles; FP64: eight, a warp's
     // last, partly filled round of FP64 tests costs as much as a full one;
     // at least one per triangle (a wing of thousands of small triangles; a
@@ -454,13 +459,13 @@ cudaError_t ps::rasterise(const MaskArgs& a, void* chi, void* us, uint8_t* flag,
     const int wpt = a.n_tri < per_sm * kRasterSM ? per_sm * kRasterSM / a.n_tri : 1;
     const int pb = (int)(((long)a.n_tri * wpt * 32 + kPairThreads - 1) / kPairThreads);
     if constexpr (sizeof(T) == 4) {
-        k_mask_pairs<T, kPairOne><<<pb, kPairThreads, 0, s>>>(m, a, np, wpt);
+        launch(k_mask_pairs<T, kPairOne>, pb, kPairThreads, 0, s, m, a, np, wpt);
     } else {
-        k_mask_pairs<T, kPairBound><<<pb, kPairThreads, 0, s>>>(m, a, np, wpt);
-        k_mask_pairs<T, kPairLeast><<<pb, kPairThreads, 0, s>>>(m, a, np, wpt);
-        k_mask_pairs<T, kPairTies><<<pb, kPairThreads, 0, s>>>(m, a, np, wpt);
+        launch(k_mask_pairs<T, kPairBound>, pb, kPairThreads, 0, s, m, a, np, wpt);
+        launch(k_mask_pairs<T, kPairLeast>, pb, kPairThreads, 0, s, m, a, np, wpt);
+        launch(k_mask_pairs<T, kPairTies>, pb, kPairThreads, 0, s, m, a, np, wpt);
     }
-    k_mask_eval<T><<<8 * kRasterSM, 256, 0, s>>>(m, a, np, (T*)chi, (T*)us, flag);
+    launch(k_mask_eval<T>, 8 * kRasterSM, 256, 0, s, m, a, np, (T*)chi, (T*)us, flag);
     *par_out = np;
     return cudaGetLastError();
 }
@@ -481,7 +486,7 @@ static cudaError_t adjoint_step_t(ps_ctx* c, const AdjW& aw, void* gchi, void* g
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_adj_spec<T>, 256, 0);
         blocks = (occ > 0 ? occ : 1) * (nsm > 0 ? nsm : 1);
     }
-    k_adj_spec<T><<<blocks, 256, 0, c->stream>>>(c->kp, (const C2*)c->adj_spec[0], (const C2*)c->adj_spec[1],
+    launch(k_adj_spec<T>, blocks, 256, 0, c->stream, c->kp, (const C2*)c->adj_spec[0], (const C2*)c->adj_spec[1],
                                                  (C2*)c->adj_spec[2], (const T*)c->b.Ex, (const T*)c->b.Ez, aw.first);
     return c->ops->adjoint(c->kp, c->b, aw, c->adj_spec[0], c->adj_spec[1], gchi, gus, c->stream);
 }
@@ -694,8 +699,8 @@ ps_status ps_set_mask(ps_ctx* c, const void* chi, const void* us) {
         return cuda_fail(c, e, "ps_set_mask copy");
     const long lines = (long)n * n;
     const int per = 8;  // lines per block (one warp each)
-    if (c->fp64) k_line_flags<double><<<(unsigned)((lines + per - 1) / per), 32 * per, 0, c->stream>>>((const double*)c->b.chi, c->b.flag, n, c->p.nz);
-    else k_line_flags<float><<<(unsigned)((lines + per - 1) / per), 32 * per, 0, c->stream>>>((const float*)c->b.chi, c->b.flag, n, c->p.nz);
+    if (c->fp64) launch(k_line_flags<double>, (unsigned)((lines + per - 1) / per), 32 * per, 0, c->stream, (const double*)c->b.chi, c->b.flag, n, c->p.nz);
+    else launch(k_line_flags<float>, (unsigned)((lines + per - 1) / per), 32 * per, 0, c->stream, (const float*)c->b.chi, c->b.flag, n, c->p.nz);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "ps_set_mask flags");
     c->mask_dense_dirty = true;
     c->has_last_mask = false;
@@ -824,9 +829,9 @@ ps_status ps_pressure_loads(ps_ctx* c, const void* p_dev, const double* xw, int3
     memcpy(a.XO, frame->X_O, sizeof(a.XO));
     const int nb = (n_nodes + kLoadWarps - 1) / kLoadWarps;
     if (c->fp64)
-        k_node_loads<double><<<nb, 32 * kLoadWarps, 0, c->stream>>>(a, (const double*)p_dev, p_nodes_dev, f_nodes_dev);
+        launch(k_node_loads<double>, nb, 32 * kLoadWarps, 0, c->stream, a, (const double*)p_dev, p_nodes_dev, f_nodes_dev);
     else
-        k_node_loads<float><<<nb, 32 * kLoadWarps, 0, c->stream>>>(a, (const float*)p_dev, p_nodes_dev, f_nodes_dev);
+        launch(k_node_loads<float>, nb, 32 * kLoadWarps, 0, c->stream, a, (const float*)p_dev, p_nodes_dev, f_nodes_dev);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "ps_pressure_loads");
     return PS_OK;
@@ -838,7 +843,7 @@ ps_status ps_forces(ps_ctx* c, double F[3], double M[3]) {
     if (c->nstep == 0) return fail(c, PS_ESTATE, "ps_forces: no step taken yet");
     DeviceGuard dg(c->device);
     const double dx = c->kp.dx;
-    k_force_final<<<6, kForceThreads, 0, c->stream>>>(c->b.partial, c->zblocks, dx * dx * dx / c->p.eta, c->b.err,
+    launch(k_force_final, 6, kForceThreads, 0, c->stream, c->b.partial, c->zblocks, dx * dx * dx / c->p.eta, c->b.err,
                                                       c->out);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "ps_forces");
@@ -915,7 +920,7 @@ ps_status ps_debug_wait_timeout(ps_ctx* c, int32_t cap) {
     if (!c) return PS_EINVAL;
     if (cap < 1) return fail(c, PS_EINVAL, "ps_debug_wait_timeout: cap < 1");
     DeviceGuard dg(c->device);
-    k_wait_timeout<<<1, 64, 0, c->stream>>>(c->b.err, (uint32_t)cap);
+    launch(k_wait_timeout, 1, 64, 0, c->stream, c->b.err, (uint32_t)cap);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "ps_debug_wait_timeout");
     return sync(c, "ps_debug_wait_timeout");
@@ -926,9 +931,9 @@ ps_status ps_diagnostics(ps_ctx* c, double* energy, double* max_div) {
     if (!energy || !max_div) return fail(c, PS_EINVAL, "ps_diagnostics: null output");
     DeviceGuard dg(c->device);
     const int nb = 304;
-    if (c->fp64) k_diag<double><<<nb, 256, 0, c->stream>>>(c->kp, (const double2*)c->b.U, c->b.partial);
-    else k_diag<float><<<nb, 256, 0, c->stream>>>(c->kp, (const float2*)c->b.U, c->b.partial);
-    k_diag_final<<<1, 32, 0, c->stream>>>(c->b.partial, nb, c->kp.half_L3, c->out + 8);
+    if (c->fp64) launch(k_diag<double>, nb, 256, 0, c->stream, c->kp, (const double2*)c->b.U, c->b.partial);
+    else launch(k_diag<float>, nb, 256, 0, c->stream, c->kp, (const float2*)c->b.U, c->b.partial);
+    launch(k_diag_final, 1, 32, 0, c->stream, c->b.partial, nb, c->kp.half_L3, c->out + 8);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "ps_diagnostics");
     double h[3];
@@ -1023,13 +1028,13 @@ ps_status ps_mask_nodes_vjp(ps_ctx* c, const void* grad_chi_dev, const void* gra
     if ((e = cudaMemsetAsync(c->gX, 0, (size_t)a.n_nodes * 3 * sizeof(double), c->stream)) != cudaSuccess)
         return cuda_fail(c, e, "ps_mask_nodes_vjp");
     if (a.profile == PS_MASK_TANH) {
-        if (c->fp64) k_mask_vjp_dense<double><<<16 * kRasterSM, 128, 0, c->stream>>>(m, a, (const double*)grad_chi_dev, (const double*)grad_us_dev, (const double*)c->b.chi, c->gX);
-        else k_mask_vjp_dense<float><<<16 * kRasterSM, 128, 0, c->stream>>>(m, a, (const float*)grad_chi_dev, (const float*)grad_us_dev, (const float*)c->b.chi, c->gX);
+        if (c->fp64) launch(k_mask_vjp_dense<double>, 16 * kRasterSM, 128, 0, c->stream, m, a, (const double*)grad_chi_dev, (const double*)grad_us_dev, (const double*)c->b.chi, c->gX);
+        else launch(k_mask_vjp_dense<float>, 16 * kRasterSM, 128, 0, c->stream, m, a, (const float*)grad_chi_dev, (const float*)grad_us_dev, (const float*)c->b.chi, c->gX);
     } else {
-        if (c->fp64) k_mask_vjp_list<double><<<8 * kRasterSM, 256, 0, c->stream>>>(m, a, c->mask_par, (const double*)grad_chi_dev, (const double*)grad_us_dev, (const double*)c->b.chi, c->gX);
-        else k_mask_vjp_list<float><<<8 * kRasterSM, 256, 0, c->stream>>>(m, a, c->mask_par, (const float*)grad_chi_dev, (const float*)grad_us_dev, (const float*)c->b.chi, c->gX);
+        if (c->fp64) launch(k_mask_vjp_list<double>, 8 * kRasterSM, 256, 0, c->stream, m, a, c->mask_par, (const double*)grad_chi_dev, (const double*)grad_us_dev, (const double*)c->b.chi, c->gX);
+        else launch(k_mask_vjp_list<float>, 8 * kRasterSM, 256, 0, c->stream, m, a, c->mask_par, (const float*)grad_chi_dev, (const float*)grad_us_dev, (const float*)c->b.chi, c->gX);
     }
-    k_vjp_to_wing<<<(a.n_nodes + 127) / 128, 128, 0, c->stream>>>(a, c->gX, grad_xw_dev);
+    launch(k_vjp_to_wing, (a.n_nodes + 127) / 128, 128, 0, c->stream, a, c->gX, grad_xw_dev);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "ps_mask_nodes_vjp");
     return PS_OK;
 }

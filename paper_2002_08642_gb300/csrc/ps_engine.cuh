@@ -159,10 +159,10 @@ template <typename T, int N, int NZ = N> struct Engine {
         const C2* tw = (const C2*)b.tw;
         if constexpr (XSPLIT) {
             const int items = kp.kyn * (KZ_ / GE::CX1) * 6;
-            k_xinv_split<T, N, KZ_><<<items < xsgrid() ? items : xsgrid(), thr_x1, sm_x1, s>>>(*b.tmU, kp, (C2*)b.A, tw,
+            launch(k_xinv_split<T, N, KZ_>, items < xsgrid() ? items : xsgrid(), thr_x1, sm_x1, s, *b.tmU, kp, (C2*)b.A, tw,
                                                                                               b.err);
         } else {
-            k_xinv_tma<T, N, 6, KZ_><<<x1grid(), thr_x1, sm_x1, s>>>(*b.tmU, kp, (C2*)b.A, tw, b.err);
+            launch(k_xinv_tma<T, N, 6, KZ_>, x1grid(), thr_x1, sm_x1, s, *b.tmU, kp, (C2*)b.A, tw, b.err);
         }
     }
     static constexpr int thr_x5 = GE::CX5 * GE::G;
@@ -247,25 +247,25 @@ template <typename T, int N, int NZ = N> struct Engine {
         if (ev) cudaEventRecord(ev[0], s);
         if (!resume) x_inverse(kp, b, s);
         if (ev) { cudaEventRecord(ev[1], s); cudaEventRecord(ev[2], s); }
-        if (!resume) k_yinv_tma<T, N, 6, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, (C2*)b.B, tw, b.err);
+        if (!resume) launch(k_yinv_tma<T, N, 6, KZ_>, y2grid(), thr_y2, sm_y2, s, *b.tmA, k1, (C2*)b.B, tw, b.err);
         if (ev) { cudaEventRecord(ev[3], s); cudaEventRecord(ev[4], s); }
         if (sp)
-            k_zpass<T, NZ, false, true, N><<<zgrid(), thr_zp, sm_zp, s>>>(k1, (C2*)b.B, (const T*)b.chi, (const T*)b.us,
+            launch(k_zpass<T, NZ, false, true, N>, zgrid(), thr_zp, sm_zp, s, k1, (C2*)b.B, (const T*)b.chi, (const T*)b.us,
                                                                      b.flag, b.partial, twz(b.tw), b.err, nullptr,
                                                                      (const T*)b.chi_sp, (C2*)b.B);
         else
-            k_zpass<T, NZ, false, false, N><<<zgrid(), thr_zp, sm_zp, s>>>(k1, (C2*)b.B, (const T*)b.chi, (const T*)b.us, b.flag,
+            launch(k_zpass<T, NZ, false, false, N>, zgrid(), thr_zp, sm_zp, s, k1, (C2*)b.B, (const T*)b.chi, (const T*)b.us, b.flag,
                                                         b.partial, twz(b.tw), b.err, nullptr, nullptr, (C2*)b.B);
         if (ev) { cudaEventRecord(ev[5], s); cudaEventRecord(ev[6], s); }
-        if (sp) k_yfwd_tma<T, N, GE::CY4, 6, KZ_><<<y4grid(), thr_y4, sm_y4, s>>>(*b.tmB, k1, (C2*)b.A, tw, b.err);
-        else k_yfwd_tma<T, N, GE::CY4, 3, KZ_><<<y4grid(), thr_y4, sm_y4, s>>>(*b.tmB, k1, (C2*)b.A, tw, b.err);
+        if (sp) launch(k_yfwd_tma<T, N, GE::CY4, 6, KZ_>, y4grid(), thr_y4, sm_y4, s, *b.tmB, k1, (C2*)b.A, tw, b.err);
+        else launch(k_yfwd_tma<T, N, GE::CY4, 3, KZ_>, y4grid(), thr_y4, sm_y4, s, *b.tmB, k1, (C2*)b.A, tw, b.err);
         if (ev) { cudaEventRecord(ev[7], s); cudaEventRecord(ev[8], s); }
         if (sp)
-            k_xfwd_tma<T, N, 0, true, KZ_><<<x5sgrid(), thr_x5, sm_x5s, s>>>(*b.tmA5, *b.tmUp, *b.tmHp, kp, (C2*)b.U,
+            launch(k_xfwd_tma<T, N, 0, true, KZ_>, x5sgrid(), thr_x5, sm_x5s, s, *b.tmA5, *b.tmUp, *b.tmHp, kp, (C2*)b.U,
                                                                        (C2*)b.H, (const T*)b.Ex, (const T*)b.Ez,
                                                                        first, tw, b.err);
         else
-            k_xfwd_tma<T, N, 0, false, KZ_><<<x5grid(), thr_x5, sm_x5t, s>>>(*b.tmA5, *b.tmUp, *b.tmHp, kp, (C2*)b.U,
+            launch(k_xfwd_tma<T, N, 0, false, KZ_>, x5grid(), thr_x5, sm_x5t, s, *b.tmA5, *b.tmUp, *b.tmHp, kp, (C2*)b.U,
                                                                 (C2*)b.H, (const T*)b.Ex, (const T*)b.Ez, first, tw,
                                                                 b.err);
         if (ev) cudaEventRecord(ev[9], s);
@@ -276,9 +276,9 @@ template <typename T, int N, int NZ = N> struct Engine {
         const C2* tw = (const C2*)b.tw;
         KP k1 = kp;
         k1.xs0 = 0; k1.xsn = N; k1.part_off = 0;
-        k_zfwd_phys<T, NZ><<<zfgrid(), thr_zf, sm_zf, s>>>(k1, (const T*)u, (C2*)b.B, twz(b.tw), b.err);
-        k_yfwd_tma<T, N, GE::CY4, 3, KZ_><<<y4grid(), thr_y4, sm_y4, s>>>(*b.tmB, k1, (C2*)b.A, tw, b.err);
-        k_xfwd_tma<T, N, 1, false, KZ_><<<x5grid(), thr_x5, sm_x5t, s>>>(*b.tmA5, *b.tmUp, *b.tmHp, k1, (C2*)b.U, (C2*)b.H,
+        launch(k_zfwd_phys<T, NZ>, zfgrid(), thr_zf, sm_zf, s, k1, (const T*)u, (C2*)b.B, twz(b.tw), b.err);
+        launch(k_yfwd_tma<T, N, GE::CY4, 3, KZ_>, y4grid(), thr_y4, sm_y4, s, *b.tmB, k1, (C2*)b.A, tw, b.err);
+        launch(k_xfwd_tma<T, N, 1, false, KZ_>, x5grid(), thr_x5, sm_x5t, s, *b.tmA5, *b.tmUp, *b.tmHp, k1, (C2*)b.U, (C2*)b.H,
                                                             (const T*)b.Ex, (const T*)b.Ez, 0, tw, b.err);
         return cudaGetLastError();
     }
@@ -287,9 +287,9 @@ template <typename T, int N, int NZ = N> struct Engine {
         const C2* tw = (const C2*)b.tw;
         KP k1 = kp;
         k1.xs0 = 0; k1.xsn = N; k1.part_off = 0;
-        k_xinv_tma<T, N, 3, KZ_><<<x1pgrid(), thr_x1, sm_x1, s>>>(*b.tmU, k1, (C2*)b.A, tw, b.err);
-        k_yinv_tma<T, N, 3, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, (C2*)b.B, tw, b.err);
-        k_zinv_phys<T, NZ><<<zigrid(), thr_zi, sm_zi, s>>>(k1, (const C2*)b.B, (T*)u, twz(b.tw), b.err);
+        launch(k_xinv_tma<T, N, 3, KZ_>, x1pgrid(), thr_x1, sm_x1, s, *b.tmU, k1, (C2*)b.A, tw, b.err);
+        launch(k_yinv_tma<T, N, 3, KZ_>, y2grid(), thr_y2, sm_y2, s, *b.tmA, k1, (C2*)b.B, tw, b.err);
+        launch(k_zinv_phys<T, NZ>, zigrid(), thr_zi, sm_zi, s, k1, (const C2*)b.B, (T*)u, twz(b.tw), b.err);
         return cudaGetLastError();
     }
 
@@ -302,15 +302,15 @@ template <typename T, int N, int NZ = N> struct Engine {
         const C2* tw = (const C2*)b.tw;
         KP k1 = kp;
         k1.xs0 = 0; k1.xsn = N; k1.part_off = 0;
-        k_xinv_tma<T, N, 3, KZ_><<<x1pgrid(), thr_x1, sm_x1, s>>>(*b.tmG, k1, (C2*)b.A, tw, b.err);
-        k_yinv_tma<T, N, 3, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, (C2*)b.NB, tw, b.err);
+        launch(k_xinv_tma<T, N, 3, KZ_>, x1pgrid(), thr_x1, sm_x1, s, *b.tmG, k1, (C2*)b.A, tw, b.err);
+        launch(k_yinv_tma<T, N, 3, KZ_>, y2grid(), thr_y2, sm_y2, s, *b.tmA, k1, (C2*)b.NB, tw, b.err);
         x_inverse(k1, b, s);
-        k_yinv_tma<T, N, 6, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, (C2*)b.B, tw, b.err);
-        k_adj_zpass<T, NZ, N><<<zagrid(), AZ::threads, AZ::smem, s>>>(k1, aw, (C2*)b.B, (const C2*)b.NB, (const T*)b.chi,
+        launch(k_yinv_tma<T, N, 6, KZ_>, y2grid(), thr_y2, sm_y2, s, *b.tmA, k1, (C2*)b.B, tw, b.err);
+        launch(k_adj_zpass<T, NZ, N>, zagrid(), AZ::threads, AZ::smem, s, k1, aw, (C2*)b.B, (const C2*)b.NB, (const T*)b.chi,
                                                                      (const T*)b.us, b.flag, (T*)gchi, (T*)gus,
                                                                      twz(b.tw), b.err);
-        k_yfwd_tma<T, N, GE::CY4, 6, KZ_><<<y4grid(), thr_y4, sm_y4, s>>>(*b.tmB, k1, (C2*)b.A, tw, b.err);
-        k_xfwd_tma<T, N, 3, true, KZ_><<<x5agrid(), thr_x5, sm_x5s, s>>>(*b.tmA5, *b.tmL, *b.tmL, k1, (C2*)lam, (C2*)mu,
+        launch(k_yfwd_tma<T, N, GE::CY4, 6, KZ_>, y4grid(), thr_y4, sm_y4, s, *b.tmB, k1, (C2*)b.A, tw, b.err);
+        launch(k_xfwd_tma<T, N, 3, true, KZ_>, x5agrid(), thr_x5, sm_x5s, s, *b.tmA5, *b.tmL, *b.tmL, k1, (C2*)lam, (C2*)mu,
                                                                        (const T*)b.Ex, (const T*)b.Ez, aw.first, tw,
                                                                        b.err);
         return cudaGetLastError();
@@ -331,19 +331,19 @@ template <typename T, int N, int NZ = N> struct Engine {
         k1.xs0 = 0; k1.xsn = N; k1.part_off = 0;
         if (!resume) {
             x_inverse(k1, b, s);
-            k_yinv_tma<T, N, 6, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, (C2*)b.B, tw, b.err);
+            launch(k_yinv_tma<T, N, 6, KZ_>, y2grid(), thr_y2, sm_y2, s, *b.tmA, k1, (C2*)b.B, tw, b.err);
         }
         C2* nout = b.N3 ? (C2*)b.N3 : (C2*)b.B;
-        k_zpass<T, NZ, true, false, N><<<zgrid(), thr_zp, sm_zp, s>>>(k1, (C2*)b.B, (const T*)b.chi, (const T*)b.us, b.flag,
+        launch(k_zpass<T, NZ, true, false, N>, zgrid(), thr_zp, sm_zp, s, k1, (C2*)b.B, (const T*)b.chi, (const T*)b.us, b.flag,
                                                           b.partial, twz(b.tw), b.err, (T*)p, nullptr, nout);
-        k_yfwd_tma<T, N, GE::CY4, 3, KZ_><<<y4grid(), thr_y4, sm_y4, s>>>(b.N3 ? *b.tmN : *b.tmB, k1, (C2*)b.A, tw,
+        launch(k_yfwd_tma<T, N, GE::CY4, 3, KZ_>, y4grid(), thr_y4, sm_y4, s, b.N3 ? *b.tmN : *b.tmB, k1, (C2*)b.A, tw,
                                                                   b.err);
         C2* pih = (C2*)b.A + (size_t)3 * N * GE::K * kp.Kzp;
-        k_xfwd_tma<T, N, 2, false, KZ_><<<x5grid(), thr_x5, sm_x5t, s>>>(*b.tmA5, *b.tmUp, *b.tmHp, k1, pih, nullptr,
+        launch(k_xfwd_tma<T, N, 2, false, KZ_>, x5grid(), thr_x5, sm_x5t, s, *b.tmA5, *b.tmUp, *b.tmHp, k1, pih, nullptr,
                                                             (const T*)b.Ex, (const T*)b.Ez, 0, tw, b.err);
-        k_xinv_tma<T, N, 1, KZ_><<<x1pgrid(), thr_x1, sm_x1, s>>>(*b.tmP, k1, (C2*)b.A, tw, b.err);
-        k_yinv_tma<T, N, 1, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, k1, nout, tw, b.err);
-        k_zinv_sub<T, NZ><<<zsgrid(), thr_zs, sm_zs, s>>>(k1, (const C2*)nout, (T*)p, twz(b.tw), b.err);
+        launch(k_xinv_tma<T, N, 1, KZ_>, x1pgrid(), thr_x1, sm_x1, s, *b.tmP, k1, (C2*)b.A, tw, b.err);
+        launch(k_yinv_tma<T, N, 1, KZ_>, y2grid(), thr_y2, sm_y2, s, *b.tmA, k1, nout, tw, b.err);
+        launch(k_zinv_sub<T, NZ>, zsgrid(), thr_zs, sm_zs, s, k1, (const C2*)nout, (T*)p, twz(b.tw), b.err);
         return cudaGetLastError();
     }
 
@@ -352,12 +352,12 @@ template <typename T, int N, int NZ = N> struct Engine {
         if (phase == 0) {
             x_inverse(kp, b, s);
         } else if (phase == 1) {
-            k_yinv_tma<T, N, 6, KZ_><<<y2grid(), thr_y2, sm_y2, s>>>(*b.tmA, kp, (C2*)b.B, tw, b.err);
-            k_zpass<T, NZ, false, false, N><<<zgrid(), thr_zp, sm_zp, s>>>(kp, (C2*)b.B, (const T*)b.chi, (const T*)b.us, b.flag,
+            launch(k_yinv_tma<T, N, 6, KZ_>, y2grid(), thr_y2, sm_y2, s, *b.tmA, kp, (C2*)b.B, tw, b.err);
+            launch(k_zpass<T, NZ, false, false, N>, zgrid(), thr_zp, sm_zp, s, kp, (C2*)b.B, (const T*)b.chi, (const T*)b.us, b.flag,
                                                         b.partial, twz(b.tw), b.err, nullptr, nullptr, (C2*)b.B);
-            k_yfwd_tma<T, N, GE::CY4, 3, KZ_><<<y4grid(), thr_y4, sm_y4, s>>>(*b.tmB, kp, (C2*)b.A, tw, b.err);
+            launch(k_yfwd_tma<T, N, GE::CY4, 3, KZ_>, y4grid(), thr_y4, sm_y4, s, *b.tmB, kp, (C2*)b.A, tw, b.err);
         } else {
-            k_xfwd_tma<T, N, 0, false, KZ_><<<x5grid(), thr_x5, sm_x5t, s>>>(*b.tmA5, *b.tmUp, *b.tmHp, kp, (C2*)b.U,
+            launch(k_xfwd_tma<T, N, 0, false, KZ_>, x5grid(), thr_x5, sm_x5t, s, *b.tmA5, *b.tmUp, *b.tmHp, kp, (C2*)b.U,
                                                                 (C2*)b.H, (const T*)b.Ex, (const T*)b.Ez, first, tw,
                                                                 b.err);
         }

@@ -557,6 +557,7 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
     constexpr int NB = GE::ZNB;
     C2* stage = reinterpret_cast<C2*>(smem_base128(smraw));   // [NB][6][LZ][KZP]
     if (smem_u32(stage) & 127u) {   // never expected: refuse to start copies
+        pdl_wait();
         if (threadIdx.x == 0) atomicExch(err, 2);
         return;
     }
@@ -585,6 +586,7 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
     }
     for (int i = threadIdx.x; i < 32 * 12; i += blockDim.x) (&wacc[0][0])[i] = 0.0;
     __syncthreads();
+    pdl_wait();
     auto issue = [&](int b, int buf) {  // one thread
         fence_proxy_async();
         mbar_arrive_expect_tx(&bar[buf], 6 * fbytes);
@@ -886,6 +888,7 @@ k_yinv_tma(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict__ 
     constexpr int NB = GE::Y2NB;
     C2* S = reinterpret_cast<C2*>(smem_base128(smraw));   // [NB][RS][CT]
     if (smem_u32(S) & 127u) {   // never expected: refuse to start copies
+        pdl_wait();
         if (threadIdx.x == 0) atomicExch(err, 2);
         return;
     }
@@ -902,6 +905,7 @@ k_yinv_tma(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict__ 
     }
     load_tw(tw, twg, GE::tw_n);
     __syncthreads();
+    pdl_wait();
     auto issue = [&](int i, int buf) {  // one thread
         const int f = i % NF, t = i / NF, x = kp.xs0 + t / NTZ, czt = t % NTZ;
         fence_proxy_async();
@@ -972,6 +976,7 @@ k_yfwd_tma(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict__ 
     extern __shared__ __align__(16) unsigned char smraw[];
     C2* S = reinterpret_cast<C2*>(smem_base128(smraw));   // [2][RS][CT]
     if (smem_u32(S) & 127u) {   // never expected: refuse to start copies
+        pdl_wait();
         if (threadIdx.x == 0) atomicExch(err, 2);
         return;
     }
@@ -988,6 +993,7 @@ k_yfwd_tma(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict__ 
     using S3 = Split3<T, N>;
     const C2* tw3 = load_tw_split<T, N>(tw, twg, GE::tw_n);
     __syncthreads();
+    pdl_wait();
     auto issue = [&](int i, int buf) {  // one thread
         const int f = i % NF, t = i / NF, x = kp.xs0 + t / NTZ, czt = t % NTZ;
         fence_proxy_async();
@@ -1072,6 +1078,7 @@ k_xinv_tma(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict__ 
     extern __shared__ __align__(16) unsigned char smraw[];
     C2* S = reinterpret_cast<C2*>(smem_base128(smraw));   // [2][RS][CT]
     if (smem_u32(S) & 127u) {
+        pdl_wait();
         if (threadIdx.x == 0) atomicExch(err, 2);
         return;
     }
@@ -1089,6 +1096,7 @@ k_xinv_tma(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict__ 
     }
     load_tw(tw, twg, GE::tw_n);
     __syncthreads();
+    pdl_wait();
     constexpr int NI = NF == 6 ? 3 : NF;   // input fields
     // load L: tile iteration L / NI, field L % NI
     auto issue = [&](int L) {  // one thread
@@ -1194,6 +1202,7 @@ k_xinv_split(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict_
     extern __shared__ __align__(16) unsigned char smraw[];
     C2* S = reinterpret_cast<C2*>(smem_base128(smraw));   // [2][RS][CT]
     if (smem_u32(S) & 127u) {
+        pdl_wait();
         if (threadIdx.x == 0) atomicExch(err, 2);
         return;
     }
@@ -1209,6 +1218,7 @@ k_xinv_split(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict_
     }
     load_tw(tw, twg, GE::tw_n);
     __syncthreads();
+    pdl_wait();
     auto addr = [&](int p) { return p * CT + col; };
     int it = 0;
     for (int i = blockIdx.x; i < NITEM; i += gridDim.x, ++it) {
@@ -1284,6 +1294,7 @@ k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUten
     extern __shared__ __align__(16) unsigned char smraw[];
     C2* S = reinterpret_cast<C2*>(smem_base128(smraw));   // [2][RS][CT]
     if (smem_u32(S) & 127u) {
+        pdl_wait();
         if (threadIdx.x == 0) atomicExch(err, 2);
         return;
     }
@@ -1305,6 +1316,7 @@ k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUten
     using S3 = Split3<T, N>;
     const C2* tw3 = load_tw_split<T, N>(tw, twg, GE::tw_n);
     __syncthreads();
+    pdl_wait();
     auto issue = [&](int L) {  // one thread
         const int t = blockIdx.x + (L / NF) * gridDim.x, f = field(L % NF), buf = L & 1;
         if (t >= NTILE) return;
@@ -1511,6 +1523,7 @@ k_zfwd_phys(KP kp, const T* __restrict__ u, cplx<T>* __restrict__ B, const cplx<
     extern __shared__ __align__(16) unsigned char smraw[];
     T* stage = reinterpret_cast<T*>(smem_base128(smraw));   // [2][3][L][N]
     if ((smem_u32(stage) & 127u) || (reinterpret_cast<uintptr_t>(u) & 15u)) {   // never expected
+        pdl_wait();
         if (threadIdx.x == 0) atomicExch(err, 2);
         return;
     }
@@ -1532,6 +1545,7 @@ k_zfwd_phys(KP kp, const T* __restrict__ u, cplx<T>* __restrict__ B, const cplx<
     }
     load_tw(tw, twg, ZP::TWN);
     __syncthreads();
+    pdl_wait();
     auto issue = [&](int b, int buf) {  // one thread
         fence_proxy_async();
         mbar_arrive_expect_tx(&bar[buf], 3 * fbytes);
@@ -1591,6 +1605,7 @@ k_zinv_phys(KP kp, const cplx<T>* __restrict__ B, T* __restrict__ u, const cplx<
     extern __shared__ __align__(16) unsigned char smraw[];
     C2* stage = reinterpret_cast<C2*>(smem_base128(smraw));   // [2][3][L][KZP]
     if (smem_u32(stage) & 127u) {   // never expected
+        pdl_wait();
         if (threadIdx.x == 0) atomicExch(err, 2);
         return;
     }
@@ -1612,6 +1627,7 @@ k_zinv_phys(KP kp, const cplx<T>* __restrict__ B, T* __restrict__ u, const cplx<
     }
     load_tw(tw, twg, ZP::TWN);
     __syncthreads();
+    pdl_wait();
     auto issue = [&](int b, int buf) {  // one thread
         fence_proxy_async();
         mbar_arrive_expect_tx(&bar[buf], 3 * fbytes);
@@ -1682,6 +1698,7 @@ k_zinv_sub(KP kp, const cplx<T>* __restrict__ B, T* __restrict__ u, const cplx<T
     C2* stage = reinterpret_cast<C2*>(smem_base128(smraw));   // [2][L][KZP] spectral
     T* ustage = reinterpret_cast<T*>(stage + 2 * L * KZP);     // [2][L][N] physical
     if ((smem_u32(stage) & 127u) || (reinterpret_cast<uintptr_t>(u) & 15u)) {   // never expected
+        pdl_wait();
         if (threadIdx.x == 0) atomicExch(err, 2);
         return;
     }
@@ -1701,6 +1718,7 @@ k_zinv_sub(KP kp, const cplx<T>* __restrict__ B, T* __restrict__ u, const cplx<T
     }
     load_tw(tw, twg, ZP::TWN);
     __syncthreads();
+    pdl_wait();
     auto issue = [&](int b, int buf) {  // one thread
         fence_proxy_async();
         mbar_arrive_expect_tx(&bar[buf], sbytes + ubytes);

@@ -13,6 +13,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "ps_async.cuh"
+
 namespace ps {
 
 struct LoadArgs {
@@ -53,6 +55,7 @@ static constexpr int kLoadWarps = 4;
 template <typename T>
 __global__ void __launch_bounds__(32 * kLoadWarps)
 k_node_loads(LoadArgs a, const T* __restrict__ pf, double* __restrict__ pn, double* __restrict__ F) {
+    pdl_wait();
     __shared__ int hit[kLoadWarps][32];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int v = blockIdx.x * kLoadWarps + wid;

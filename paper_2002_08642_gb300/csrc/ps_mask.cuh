@@ -49,6 +49,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "ps_async.cuh"
+
 #include <string>
 
 namespace ps {
@@ -288,6 +290,7 @@ __device__ __forceinline__ void tri_setup(const MaskWs& m, const MaskArgs& a, in
 template <typename T, bool BAND>
 __global__ void k_mask_prepare(MaskWs m, MaskArgs a, int par, T* chi, T* us, uint8_t* flag, size_t n3, size_t nflag,
                                double reach) {
+    pdl_wait();
     const unsigned long long tid = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned long long nth = (unsigned long long)gridDim.x * blockDim.x;
     if (tid == 0) m.cnt[par ^ 1] = 0;
@@ -330,6 +333,7 @@ static constexpr int kPairThreads = 256;
 enum PairWalk { kPairOne, kPairBound, kPairLeast, kPairTies };
 template <typename T, int WALK>
 __global__ void __launch_bounds__(kPairThreads) k_mask_pairs(MaskWs m, MaskArgs a, int par, int wpt) {
+    pdl_wait();
     const uint32_t warp = (blockIdx.x * (uint32_t)kPairThreads + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     const int t = (int)(warp / (uint32_t)wpt);
@@ -508,6 +512,7 @@ __device__ __forceinline__ void eval_point(const MaskWs& m, const MaskArgs& a, u
 
 template <typename T>
 __global__ void k_mask_eval(MaskWs m, MaskArgs a, int par, T* chi, T* us, uint8_t* flag) {
+    pdl_wait();
     const unsigned long long cnt = m.cnt[par];
     const uint32_t* const list = par ? m.list[1] : m.list[0];
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
@@ -527,6 +532,7 @@ __global__ void k_mask_eval(MaskWs m, MaskArgs a, int par, T* chi, T* us, uint8_
 // Dense (tanh) profile: every point against every triangle in index order.
 template <typename T>
 __global__ void k_mask_dense(MaskWs m, MaskArgs a, T* chi, T* us, uint8_t* flag) {
+    pdl_wait();
     const size_t n = a.n, nz = a.nz, n3 = n * n * nz;
     for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < n3; p += (size_t)gridDim.x * blockDim.x) {
         const int k = (int)(p % nz), j = (int)((p / nz) % n), i = (int)(p / (n * nz));
