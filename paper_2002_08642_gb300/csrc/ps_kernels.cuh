@@ -45,6 +45,9 @@
 #ifndef PS_ZP_SMEM_KB
 #define PS_ZP_SMEM_KB 100
 #endif
+#ifndef PS_ZSHORT
+#define PS_ZSHORT 768
+#endif
 #ifndef PS_ZP_MINB
 #define PS_ZP_MINB 0   // 0: automatic (Geo::ZMINB)
 #endif
@@ -216,10 +219,13 @@ template <typename T, int N> struct Geo {
     }
     static constexpr int LZ = lz_pick();
     // three blocks per SM where the register cap this sets (<= 72 at 288
-    // threads) costs no more than a few spilled words, else two; never more
-    // than the shared memory lets reside
+    // threads) costs no more than a few spilled words, else two; short FP32
+    // lines (blocks of at most 96 threads): 768 threads per SM, 80 registers
+    // without spills (left to itself the compiler takes 115); never more than
+    // the shared memory lets reside
     static constexpr int ZFIT = (227 * 1024) / (zsmem(LZ) + 4096) > 0 ? (227 * 1024) / (zsmem(LZ) + 4096) : 1;
-    static constexpr int ZMIN0 = (3 * LZ * G <= 288 || N <= 256) ? 3 : 2;
+    static constexpr int ZTHR = (3 * LZ * G + 31) / 32 * 32;
+    static constexpr int ZMIN0 = sizeof(T) == 4 && ZTHR <= 96 ? PS_ZSHORT / ZTHR : (3 * LZ * G <= 288 || N <= 256) ? 3 : 2;
     static constexpr int ZMINB = PS_ZP_MINB > 0 ? PS_ZP_MINB : (ZMIN0 < ZFIT ? ZMIN0 : ZFIT);
     // TMA-staged y passes: K = kept x/y modes; inputs come in boxes of at
     // most 256 rows (NBOX boxes of BR rows cover R rows)
@@ -666,8 +672,9 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
         using Sum = typename sum_of<T>::type;
         Sum fm[6] = {};   // q and (offset from jc in cells) x q
         bool touched = false;
-        // n = u x w - (chi/eta)(u - us) of line l at z and the force sums
-        auto nonlinear = [&](int l, int z, int a, T& nx, T& ny, T& nz) {
+        // n = u x w - (chi/eta)(u - us) of line l at z and the force sums;
+        // cs: chi and us there if the line is flagged
+        auto nonlinear = [&](int l, int z, int a, const T* cs, T& nx, T& ny, T& nz) {
             const long lid = (long)b * LZ + l;
             const C2 z0 = tile(l, 0)[a], z1 = tile(l, 1)[a], z2 = tile(l, 2)[a];
             const T ux = z0.x, uy = z0.y, uz = z1.x, wx = z1.y, wy = z2.x, wz = z2.y;
@@ -676,11 +683,10 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
             nz = ux * wy - uy * wx;
             if constexpr (PM) half_u2[(size_t)lid * N + z] = (T)0.5 * (ux * ux + uy * uy + uz * uz);
             if (sflag[l] != 0) {
-                const size_t po = (size_t)lid * N + z;
-                const T c = chi[po];
+                const T c = cs[0];
                 if (c != (T)0) {
                     const int x = (int)(lid / nyl), y = (int)(lid % nyl);
-                    const T sx = us[po], sy = us[N3 + po], sz = us[2 * N3 + po];
+                    const T sx = cs[1], sy = cs[2], sz = cs[3];
                     const T ce = c * inv_eta;
                     nx -= ce * (ux - sx);
                     ny -= ce * (uy - sy);
@@ -710,9 +716,24 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
             // tile position r holds z = r (n = 3M: z = 3 (r mod M) + r / M)
             const int z = Z3 ? 3 * (r % M) + r / M : r;
             const int a = zad(r);
+            // mask and solid velocity of the flagged lines: all eight loads at
+            // once (one memory latency per round, also where chi turns out 0;
+            // loading u_s after chi, line after line, took four; with the
+            // register budget of short lines: plate 128^3 805 -> 758 us,
+            // wing 256^3 2164 -> 2136)
+            T cs[2][4];
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                if (sflag[l + j] != 0) {
+                    const size_t po = ((size_t)b * LZ + l + j) * N + z;
+                    cs[j][0] = chi[po];
+                    cs[j][1] = us[po];
+                    cs[j][2] = us[N3 + po];
+                    cs[j][3] = us[2 * N3 + po];
+                }
             T nx0, ny0, nz0, nx1, ny1, nz1;
-            nonlinear(l, z, a, nx0, ny0, nz0);
-            nonlinear(l + 1, z, a, nx1, ny1, nz1);
+            nonlinear(l, z, a, cs[0], nx0, ny0, nz0);
+            nonlinear(l + 1, z, a, cs[1], nx1, ny1, nz1);
             if constexpr (SP) {
                 // s = chi_sp omega of both lines, read before their slots are reused
                 const long lid0 = (long)b * LZ + l;
