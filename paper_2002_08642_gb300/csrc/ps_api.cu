@@ -451,19 +451,21 @@ cudaError_t ps::rasterise(const MaskArgs& a, void* chi, void* us, uint8_t* flag,
         return cudaGetLastError();
     }
     launch(k_mask_prepare<T, true>, cb, 256, 0, s, m, a, par, (T*)chi, (T*)us, flag, n3, n * n, a.tw + a.h);
-    // FP32: about 32 warps per SM over the triangles; FP64: eight, a warp's
-    // last, partly filled round of FP64 tests costs as much as a full one;
-    // at least one per triangle (a wing of thousands of small triangles; a
-    // plate of two large ones is split finely)
-    const int per_sm = sizeof(T) == 4 ? 32 : 8;
-    const int wpt = a.n_tri < per_sm * kRasterSM ? per_sm * kRasterSM / a.n_tri : 1;
-    const int pb = (int)(((long)a.n_tri * wpt * 32 + kPairThreads - 1) / kPairThreads);
+    // about 32 warps per SM over the triangles for FP32 walks; eight for the
+    // FP64 ones, where a warp's last, partly filled round of tests costs as
+    // much as a full one; at least one per triangle (a wing of thousands of
+    // small triangles; a plate of two large ones is split finely)
+    auto walk = [&](auto kernel, int per_sm) {
+        const int wpt = a.n_tri < per_sm * kRasterSM ? per_sm * kRasterSM / a.n_tri : 1;
+        const int pb = (int)(((long)a.n_tri * wpt * 32 + kPairThreads - 1) / kPairThreads);
+        launch(kernel, pb, kPairThreads, 0, s, m, a, np, wpt);
+    };
     if constexpr (sizeof(T) == 4) {
-        launch(k_mask_pairs<T, kPairOne>, pb, kPairThreads, 0, s, m, a, np, wpt);
+        walk(k_mask_pairs<T, kPairOne>, 32);
     } else {
-        launch(k_mask_pairs<T, kPairBound>, pb, kPairThreads, 0, s, m, a, np, wpt);
-        launch(k_mask_pairs<T, kPairLeast>, pb, kPairThreads, 0, s, m, a, np, wpt);
-        launch(k_mask_pairs<T, kPairTies>, pb, kPairThreads, 0, s, m, a, np, wpt);
+        walk(k_mask_pairs<T, kPairBound>, 32);
+        walk(k_mask_pairs<T, kPairLeast>, 8);
+        walk(k_mask_pairs<T, kPairTies>, 8);
     }
     launch(k_mask_eval<T>, 8 * kRasterSM, 256, 0, s, m, a, np, (T*)chi, (T*)us, flag);
     *par_out = np;

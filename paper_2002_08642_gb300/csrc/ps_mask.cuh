@@ -12,8 +12,8 @@
 // Banded (cosine) profile, three kernels per call (five in FP64):
 //   prepare   zero chi/u_s and reset the per-point keys of the points the
 //             previous call touched (list kept in the workspace), clear the
-//             line flags; the global node positions X_O + R x^(w) (double);
-//             per triangle the grid-index bounding box and the geometry the
+//             line flags; the global node positions X_O + R x^(w) and
+//             velocities R v^(w) (double); per triangle the grid-index bounding box and the geometry the
 //             pair tests need, in the context precision;
 //   pairs     a warp per triangle (several where there are few) walks the
 //             points of its box. FP32: for every pair with distance < reach
@@ -93,7 +93,7 @@ static_assert(sizeof(TriGeo<double>) <= kTriGeoBytes, "triangle geometry slot");
 inline size_t mask_workspace_bytes(int n, int nz) {
     const size_t n3 = (size_t)n * n * nz;
     auto a = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    return a(n3 * 8) + a(n3 * 4) + 2 * a(n3 * 4) + a(64) + a((size_t)kMaskMaxNodes * 3 * 8) +
+    return a(n3 * 8) + a(n3 * 4) + 2 * a(n3 * 4) + a(64) + 2 * a((size_t)kMaskMaxNodes * 3 * 8) +
            a((size_t)kMaskMaxTri * kTriGeoBytes);
 }
 
@@ -102,7 +102,8 @@ struct MaskWs {
     int32_t* win;
     uint32_t* list[2];
     unsigned long long* cnt;  // [0],[1]: list lengths, [4]: bad-index flag
-    double* xg;
+    double* xg;                // node positions, global
+    double* vg;                // R times the wing-frame node velocities
     unsigned char* geo;        // per triangle: TriGeo<T> in kTriGeoBytes
 };
 
@@ -117,6 +118,7 @@ inline MaskWs mask_ws_split(unsigned char* w, int n, int nz) {
     m.list[1] = (uint32_t*)(w + o); o += a(n3 * 4);
     m.cnt = (unsigned long long*)(w + o); o += a(64);
     m.xg = (double*)(w + o); o += a((size_t)kMaskMaxNodes * 3 * 8);
+    m.vg = (double*)(w + o); o += a((size_t)kMaskMaxNodes * 3 * 8);
     m.geo = w + o;
     return m;
 }
@@ -169,6 +171,14 @@ __device__ __forceinline__ R closest_tri(const R p[3], const R a[3], const R b[3
     return d2s;
 }
 
+// x <= 0 and x >= 0 of a number that is no NaN, on the integer pipe for
+// doubles (a -0 counts as below 0 in ge0: a region's boundary, either side of
+// which gives the same point).
+__device__ __forceinline__ bool le0(float x) { return x <= 0.0f; }
+__device__ __forceinline__ bool ge0(float x) { return x >= 0.0f; }
+__device__ __forceinline__ bool le0(double x) { return __double_as_longlong(x) <= 0; }
+__device__ __forceinline__ bool ge0(double x) { return __double2hiint(x) >= 0; }
+
 // Barycentrics (v of b, w of c) of the point of the triangle (0, b, c) closest
 // to P, by the same region tests as closest_tri with the dot products
 // relative to vertex a: bp = P - b and cp = P - c enter through
@@ -177,22 +187,23 @@ template <typename R>
 __device__ __forceinline__ void closest_rel(const R P[3], const R b[3], const R c[3], R bb, R bc, R cc, R& v, R& w) {
     const R d1 = b[0] * P[0] + b[1] * P[1] + b[2] * P[2];
     const R d2 = c[0] * P[0] + c[1] * P[1] + c[2] * P[2];
-    if (d1 <= (R)0 && d2 <= (R)0) { v = 0; w = 0; return; }
+    if (le0(d1) && le0(d2)) { v = 0; w = 0; return; }
     const R d3 = d1 - bb, d4 = d2 - bc, d5 = d1 - bc, d6 = d2 - cc;
-    if (d3 >= (R)0 && d4 <= d3) { v = 1; w = 0; return; }
-    if (d6 >= (R)0 && d5 <= d6) { v = 0; w = 1; return; }
+    const R d43 = d4 - d3, d56 = d5 - d6;
+    if (ge0(d3) && le0(d43)) { v = 1; w = 0; return; }
+    if (ge0(d6) && le0(d56)) { v = 0; w = 1; return; }
     const R vc = d1 * d4 - d3 * d2;
     const R vb = d5 * d2 - d1 * d6;
     const R va = d3 * d6 - d5 * d4;
     // one division for all remaining regions: an edge's or the face's parameter
-    const bool e_ab = vc <= (R)0 && d1 >= (R)0 && d3 <= (R)0;
-    const bool e_ac = !e_ab && vb <= (R)0 && d2 >= (R)0 && d6 <= (R)0;
-    const bool e_bc = !e_ab && !e_ac && va <= (R)0 && (d4 - d3) >= (R)0 && (d5 - d6) >= (R)0;
-    const R den = e_ab ? d1 - d3 : e_ac ? d2 - d6 : e_bc ? (d4 - d3) + (d5 - d6) : va + vb + vc;
+    const bool e_ab = le0(vc) && ge0(d1) && le0(d3);
+    const bool e_ac = !e_ab && le0(vb) && ge0(d2) && le0(d6);
+    const bool e_bc = !e_ab && !e_ac && le0(va) && ge0(d43) && ge0(d56);
+    const R den = e_ab ? d1 - d3 : e_ac ? d2 - d6 : e_bc ? d43 + d56 : va + vb + vc;
     const R q = (R)1 / den;
     if (e_ab) { v = d1 * q; w = 0; }
     else if (e_ac) { v = 0; w = d2 * q; }
-    else if (e_bc) { w = (d4 - d3) * q; v = (R)1 - w; }
+    else if (e_bc) { w = d43 * q; v = (R)1 - w; }
     else { v = vb * q; w = vc * q; }
 }
 
@@ -297,9 +308,13 @@ __global__ void k_mask_prepare(MaskWs m, MaskArgs a, int par, T* chi, T* us, uin
     if (tid < (unsigned long long)a.n_nodes) {
         const int i = (int)tid;
         for (int r = 0; r < 3; ++r) {
-            double s = a.XO[r];
-            for (int c = 0; c < 3; ++c) s += a.R[3 * r + c] * a.xw[3 * i + c];
+            double s = a.XO[r], v = 0.0;
+            for (int c = 0; c < 3; ++c) {
+                s += a.R[3 * r + c] * a.xw[3 * i + c];
+                v += a.R[3 * r + c] * a.vw[3 * i + c];
+            }
             m.xg[3 * i + r] = s;
+            m.vg[3 * i + r] = v;
         }
     }
     if constexpr (BAND) {
@@ -326,6 +341,17 @@ __global__ void k_mask_prepare(MaskWs m, MaskArgs a, int par, T* chi, T* us, uin
 // Tolerance of near-ties of squared distances (FP64): 4 units in the last
 // place of the distance (the same pair recomputed may round differently).
 __device__ __forceinline__ double tie_limit(double d2) { return d2 + (d2 * 1.8e-15 + 1e-300); }
+
+// Bits of the double equal to a normal float > 0, and the float at or just
+// below a double given by its bits (0 below the float range, its end above):
+// on the integer pipe, a conversion takes 64 cycles like any FP64 instruction.
+__device__ __forceinline__ unsigned long long widen(float x) {
+    return ((unsigned long long)__float_as_uint(x) << 29) + (896ull << 52);
+}
+__device__ __forceinline__ float narrow(unsigned long long bits) {
+    const long long e = (long long)(bits >> 29) - (896ll << 23);
+    return __int_as_float(e < 0 ? 0 : e > 0x7f7fffffll ? 0x7f7fffff : (int)e);
+}
 
 // Warp (t, part) of wpt per triangle: points 32 part .. 32 part + 31 of
 // triangle t's box, and on by 32 wpt.
@@ -407,8 +433,8 @@ __global__ void __launch_bounds__(kPairThreads) k_mask_pairs(MaskWs m, MaskArgs 
                     const float q = P[r] - v * b[r] - w * c[r];
                     s += q * q;
                 }
-                const double up = (double)(sqrtf(s) + err);
-                offer(index(i, j, k), (unsigned long long)__double_as_longlong(up * up));
+                const float up = sqrtf(s) + err;
+                offer(index(i, j, k), widen(fmaxf(up * up * 1.00001f, 1e-37f)));
             }
         } else {
             const double reach2 = reach * reach;
@@ -440,7 +466,7 @@ __global__ void __launch_bounds__(kPairThreads) k_mask_pairs(MaskWs m, MaskArgs 
                     const float lo = lower(P);
                     // at most the least distance so far, with the tie's margin
                     const unsigned long long key = __ldcg(&m.key[index(i, j, k)]);
-                    in = lo <= freach && lo * lo <= (float)__longlong_as_double((long long)key) * 1.0001f;
+                    in = lo <= freach && lo * lo <= narrow(key) * 1.0001f + 2e-37f;
                 }
                 const unsigned b = __ballot_sync(0xffffffffu, in);
                 if (in) Q[nq + __popc(b & ((1u << lane) - 1u))] = l;
@@ -457,11 +483,29 @@ __global__ void __launch_bounds__(kPairThreads) k_mask_pairs(MaskWs m, MaskArgs 
     }
 }
 
+// sin(pi s), |s| <= 1/2: its series to s^21 (the next term is below 1e-17
+// there); half the FP64 instructions of cospi with its range reduction.
+__device__ __forceinline__ double sin_pi_half(double s) {
+    const double q = s * s;
+    double r = 5.39266466260812895e-10;
+    r = fma(r, q, -2.29484289972698730e-08);
+    r = fma(r, q, 7.95205400147551261e-07);
+    r = fma(r, q, -2.19153534478302173e-05);
+    r = fma(r, q, 4.66302805767612554e-04);
+    r = fma(r, q, -7.37043094571435044e-03);
+    r = fma(r, q, 8.21458866111282326e-02);
+    r = fma(r, q, -5.99264529320792105e-01);
+    r = fma(r, q, 2.55016403987734552e+00);
+    r = fma(r, q, -5.16771278004997026e+00);
+    r = fma(r, q, 3.14159265358979312e+00);
+    return r * s;
+}
+
 __device__ __forceinline__ double chi_profile(double d, double tw, double h, int profile) {
     if (profile == 1) return 0.5 * (1.0 - tanh((d - tw) / h));
     if (d <= tw - h) return 1.0;
     if (d >= tw + h) return 0.0;
-    return 0.5 * (1.0 + cospi((d - tw + h) * (0.5 / h)));
+    return 0.5 - 0.5 * sin_pi_half((d - tw) * (0.5 / h));   // = (1 + cos(pi (d - tw + h) / (2 h))) / 2
 }
 
 // chi and u_s at grid point p from triangle t (double throughout).
@@ -493,17 +537,13 @@ __device__ __forceinline__ void eval_point(const MaskWs& m, const MaskArgs& a, u
     const double chi_p = chi_profile(sqrt(d2), a.tw, a.h, a.profile);
     chi[p] = (T)chi_p;
     if (chi_p > 0.0 || a.profile == 1) {
+        // u_s = V_O + Omega x (x - X_O) + sum beta R v
         const double u = 1.0 - v - w;
-        double vl[3], rr[3];
+        const double rr[3] = {X[0] - a.XO[0], X[1] - a.XO[1], X[2] - a.XO[2]};
         for (int r = 0; r < 3; ++r) {
-            vl[r] = u * a.vw[3 * id[0] + r] + v * a.vw[3 * id[1] + r] + w * a.vw[3 * id[2] + r];
-            rr[r] = X[r] - a.XO[r];
-        }
-        const double rot[3] = {a.Om[1] * rr[2] - a.Om[2] * rr[1], a.Om[2] * rr[0] - a.Om[0] * rr[2],
-                               a.Om[0] * rr[1] - a.Om[1] * rr[0]};
-        for (int r = 0; r < 3; ++r) {
-            double g = a.VO[r] + rot[r];
-            for (int q = 0; q < 3; ++q) g += a.R[3 * r + q] * vl[q];
+            const int r1 = (r + 1) % 3, r2 = (r + 2) % 3;
+            double g = a.VO[r] + a.Om[r1] * rr[r2] - a.Om[r2] * rr[r1];
+            g += u * m.vg[3 * id[0] + r] + v * m.vg[3 * id[1] + r] + w * m.vg[3 * id[2] + r];
             us[r * n3 + p] = (T)g;
         }
         if (chi_p > 0.0) flag[line] = 1;
