@@ -210,7 +210,14 @@ template <typename T, int N> struct Geo {
     // 256^3 z pass 0.187 -> 0.177 ms); longer lines the largest batch within
     // the thread and shared-memory budgets (384^3: 0.611 ms against 0.652 ms
     // with 2 lines)
+    // FP64 (an instruction costs a warp the same however many of its lanes are
+    // there): the smallest batch of up to 8 lines of one x-plane that fills
+    // whole warps, if there is one (128^3: 96 threads for 4 lines instead of
+    // 48 for 2; FP64 wing at 128^3 2896 -> 2687 us)
     static constexpr int lz_pick() {
+        if (sizeof(T) == 8)
+            for (int l = 2; l <= 8; l *= 2)
+                if (3 * l * G % 32 == 0 && 3 * l * G <= 96 && N % l == 0 && zsmem(l) <= PS_ZP_SMEM_KB * 1024) return l;
         const int maxthr = G <= 16 ? 6 * G : PS_ZP_MAXTHR;
         int l = 2;
         while (3 * (2 * l) * G <= maxthr && zsmem(2 * l) <= PS_ZP_SMEM_KB * 1024 && (N * N) % (2 * l) == 0)
@@ -778,10 +785,13 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
         }
         __syncthreads();
         {
-            // forward lines: (l, 0) for every l, (l, 1) for even l; others idle
-            // (with the sponge: every tile)
-            const bool active = SP || (pr == 0) || (pr == 1 && (pl & 1) == 0);
-            const int tbase = (int)(tile(pl, SP ? pr : (pr == 2 ? 1 : pr)) - tiles);
+            // forward lines: (l, 0) for every l, (l, 1) for even l, by the
+            // first groups; the rest (whole warps of them) idle. With the
+            // sponge every tile
+            constexpr int NJ = SP ? 3 * LZ : LZ + LZ / 2;
+            const bool active = fl < NJ;
+            const int jl = SP ? pl : fl < LZ ? fl : active ? 2 * (fl - LZ) : 0, jp = SP ? pr : fl < LZ ? 0 : 1;
+            const int tbase = (int)(tile(jl, jp) - tiles);
             auto noload = [&](int) -> C2 { return cmk<C2>((T)0, (T)0); };
             if constexpr (Z3) {
                 const int sub = g / GM, gm = g % GM;
