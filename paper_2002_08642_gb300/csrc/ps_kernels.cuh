@@ -206,21 +206,24 @@ template <typename T, int N> struct Geo {
     static constexpr int zsmem(int l) {
         return (int)sizeof(C2) * (ZNB * 6 * l * KZP + 3 * l * LP + tw_count(N, RM) + 1) + 128;
     }
-    // lines of at most 16 threads take batches of 2 lines (measured on GB300:
-    // 256^3 z pass 0.187 -> 0.177 ms); longer lines the largest batch within
-    // the thread and shared-memory budgets (384^3: 0.611 ms against 0.652 ms
-    // with 2 lines)
-    // FP64 (an instruction costs a warp the same however many of its lanes are
-    // there): the smallest batch of up to 8 lines of one x-plane that fills
-    // whole warps, if there is one (128^3: 96 threads for 4 lines instead of
-    // 48 for 2; FP64 wing at 128^3 2896 -> 2687 us)
+    // Lines of at most 16 threads: the smallest batch that fills whole warps
+    // (a partial warp's instructions cost as much as a whole one's; FP64
+    // 128^3, 96 threads for 4 lines instead of 48 for 2: wing 2896 -> 2687 us;
+    // FP32 128^3 plate run 756 -> 708, 384^2 x 192 box 2315 -> 2230), of lines of
+    // one x-plane, up to 288 threads (FP64: 96), that leaves eight blocks per SM
+    // (FP32; 48^3 with 288-thread blocks 628 -> 650 us); else two lines.
+    // Longer lines: the largest batch within the thread and shared-memory
+    // budgets (384^3: 0.611 ms against 0.652 ms with 2 lines)
     static constexpr int lz_pick() {
-        if (sizeof(T) == 8)
-            for (int l = 2; l <= 8; l *= 2)
-                if (3 * l * G % 32 == 0 && 3 * l * G <= 96 && N % l == 0 && zsmem(l) <= PS_ZP_SMEM_KB * 1024) return l;
-        const int maxthr = G <= 16 ? 6 * G : PS_ZP_MAXTHR;
+        if (G <= 16) {
+            for (int l = 2; l <= 16; l *= 2)
+                if (3 * l * G % 32 == 0 && 3 * l * G <= (sizeof(T) == 8 ? 96 : 288) && N % l == 0 &&
+                    zsmem(l) <= PS_ZP_SMEM_KB * 1024 && (sizeof(T) == 8 || N * N / l >= 8 * 152))
+                    return l;
+            return 2;
+        }
         int l = 2;
-        while (3 * (2 * l) * G <= maxthr && zsmem(2 * l) <= PS_ZP_SMEM_KB * 1024 && (N * N) % (2 * l) == 0)
+        while (3 * (2 * l) * G <= PS_ZP_MAXTHR && zsmem(2 * l) <= PS_ZP_SMEM_KB * 1024 && (N * N) % (2 * l) == 0)
             l *= 2;
         return l;
     }
