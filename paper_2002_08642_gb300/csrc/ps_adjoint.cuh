@@ -70,90 +70,87 @@ __device__ __forceinline__ double chi_profile_d(double d, double tw, double h, i
         return -0.5 * (1.0 - t * t) / h;
     }
     if (d <= tw - h || d >= tw + h) return 0.0;
-    return -0.25 * M_PI / h * sin(M_PI * (d - tw + h) / (2.0 * h));
+    const double t = (d - tw + h) * (0.5 / h);   // -(pi / 4 h) sin(pi t), 0 < t < 1
+    return -0.25 * M_PI / h * sin_pi_half(t <= 0.5 ? t : 1.0 - t);
 }
 
 // One grid point p with closest triangle t: dJ/dX (global vertex positions)
 // accumulated into gX with atomics. The closest triangle is held fixed; the
 // distance derivative is -beta_v (p - q)/delta (envelope theorem), the
 // barycentric weights are differentiated on their active face.
+// One chain of FP64 instructions per point (64 cycles each): positions
+// relative to vertex 0, the node velocities rotated beforehand, an edge's two
+// vertices picked by selects instead of indexed local arrays (GB300, wing at
+// 64^3 FP64: 48 -> 27 us per call).
 template <typename T>
 __device__ void vjp_point(const MaskWs& m, const MaskArgs& a, uint32_t p, int t, const T* __restrict__ gchi,
                           const T* __restrict__ gus, const T* __restrict__ chi, double* __restrict__ gX) {
-    const size_t n = a.n, nz = a.nz, n3 = n * n * nz;
-    const int k = (int)(p % nz), j = (int)((p / nz) % n), i = (int)(p / (n * nz));
-    const double P[3] = {i * a.dx, j * a.dx, k * a.dx};
+    const uint32_t un = (uint32_t)a.n, unz = (uint32_t)a.nz, line = p / unz, i = line / un;
+    const size_t n3 = (size_t)un * un * unz;
+    const double X[3] = {(int)i * a.dx, (int)(line - i * un) * a.dx, (int)(p - line * unz) * a.dx};
     const int id[3] = {a.tri[3 * t], a.tri[3 * t + 1], a.tri[3 * t + 2]};
-    double X[3][3];
-    for (int v = 0; v < 3; ++v)
-        for (int r = 0; r < 3; ++r) X[v][r] = m.xg[3 * id[v] + r];
-    double Pr[3], V[3][3];
+    double P[3], e1[3], e2[3], m00 = 0.0, m01 = 0.0, m11 = 0.0;   // point and vertices 1, 2 relative to vertex 0
     for (int r = 0; r < 3; ++r) {
-        Pr[r] = P[r] - X[0][r];
-        V[0][r] = 0.0;
-        V[1][r] = X[1][r] - X[0][r];
-        V[2][r] = X[2][r] - X[0][r];
+        const double x0 = m.xg[3 * id[0] + r];
+        P[r] = X[r] - x0;
+        e1[r] = m.xg[3 * id[1] + r] - x0;
+        e2[r] = m.xg[3 * id[2] + r] - x0;
+        m00 += e1[r] * e1[r];
+        m01 += e1[r] * e2[r];
+        m11 += e2[r] * e2[r];
     }
-    double beta[3];
-    const double d = sqrt(closest_tri<double>(Pr, V[0], V[1], V[2], beta));
-    double q[3];
-    for (int r = 0; r < 3; ++r) q[r] = beta[0] * X[0][r] + beta[1] * X[1][r] + beta[2] * X[2][r];
+    double s_, t_, q[3], d2 = 0.0;
+    closest_rel<double>(P, e1, e2, m00, m01, m11, s_, t_);
+    const double u_ = 1.0 - s_ - t_;
+    for (int r = 0; r < 3; ++r) {
+        q[r] = P[r] - s_ * e1[r] - t_ * e2[r];
+        d2 += q[r] * q[r];
+    }
+    const double d = sqrt(d2);
     double acc[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
     const double cb = (double)gchi[p];
     if (d > 0.0 && cb != 0.0) {
-        const double gd = cb * chi_profile_d(d, a.tw, a.h, a.profile);
-        for (int v = 0; v < 3; ++v)
-            for (int r = 0; r < 3; ++r) acc[v][r] += gd * (-beta[v] * (P[r] - q[r]) / d);
+        const double gd = -cb * chi_profile_d(d, a.tw, a.h, a.profile) / d;
+        for (int r = 0; r < 3; ++r) {
+            const double f = gd * q[r];
+            acc[0][r] = f * u_;
+            acc[1][r] = f * s_;
+            acc[2][r] = f * t_;
+        }
     }
     const bool has_us = (a.profile == 1) || (double)chi[p] > 0.0;
     if (has_us) {
-        const double ub[3] = {(double)gus[p], (double)gus[n3 + p], (double)gus[2 * n3 + p]};
-        double g[3];
-        for (int v = 0; v < 3; ++v) {   // dJ/dbeta_v = ub . (R vw_v)
-            double s = 0.0;
-            for (int r = 0; r < 3; ++r) {
-                double rv = 0.0;
-                for (int c = 0; c < 3; ++c) rv += a.R[3 * r + c] * a.vw[3 * id[v] + c];
-                s += ub[r] * rv;
-            }
-            g[v] = s;
+        double g[3] = {0.0, 0.0, 0.0};   // dJ/dbeta_v = (dJ/du_s) . (R vw_v)
+        for (int r = 0; r < 3; ++r) {
+            const double ub = (double)gus[r * n3 + p];
+            for (int v = 0; v < 3; ++v) g[v] += ub * m.vg[3 * id[v] + r];
         }
-        int na = 0, act[3];
-        for (int v = 0; v < 3; ++v)
-            if (beta[v] > 1e-12) act[na++] = v;
-        if (na == 2) {
-            const int iu = act[0], iv = act[1];
-            double e[3], pu[3];
-            double dd = 0.0, nn = 0.0;
+        const bool on0 = u_ > 1e-12, on1 = s_ > 1e-12, on2 = t_ > 1e-12;
+        const int na = (int)on0 + (int)on1 + (int)on2;
+        if (na == 2) {   // edge from vertex iu to iv > iu: iu = 0 if on0 else 1, iv = 2 if on2 else 1
+            double e[3], pu[3], dd = 0.0, nn = 0.0;
             for (int r = 0; r < 3; ++r) {
-                e[r] = X[iv][r] - X[iu][r];
-                pu[r] = P[r] - X[iu][r];
+                const double xu = on0 ? 0.0 : e1[r], xv = on2 ? e2[r] : e1[r];
+                e[r] = xv - xu;
+                pu[r] = P[r] - xu;
                 dd += e[r] * e[r];
                 nn += pu[r] * e[r];
             }
-            const double gt = g[iv] - g[iu];
+            const double gt = ((on2 ? g[2] : g[1]) - (on0 ? g[0] : g[1])) / (dd * dd), n2 = 2.0 * nn;
             for (int r = 0; r < 3; ++r) {
-                acc[iu][r] += gt * ((-(e[r] + pu[r]) * dd + 2.0 * nn * e[r]) / (dd * dd));
-                acc[iv][r] += gt * ((pu[r] * dd - 2.0 * nn * e[r]) / (dd * dd));
+                const double fv = gt * (pu[r] * dd - n2 * e[r]);
+                const double fu = gt * (n2 * e[r] - (e[r] + pu[r]) * dd);
+                if (on0) acc[0][r] += fu; else acc[1][r] += fu;
+                if (on2) acc[2][r] += fv; else acc[1][r] += fv;
             }
         } else if (na == 3) {
-            const double* e0 = V[1];
-            const double* e1 = V[2];
-            const double* dv = Pr;
-            const double s_ = beta[1], t_ = beta[2];
-            double m00 = 0, m01 = 0, m11 = 0;
-            for (int r = 0; r < 3; ++r) {
-                m00 += e0[r] * e0[r];
-                m01 += e0[r] * e1[r];
-                m11 += e1[r] * e1[r];
-            }
             const double g0 = g[1] - g[0], g1 = g[2] - g[0];
-            const double det = m00 * m11 - m01 * m01;
-            const double z0 = (m11 * g0 - m01 * g1) / det, z1 = (m00 * g1 - m01 * g0) / det;
+            const double idet = 1.0 / (m00 * m11 - m01 * m01);
+            const double z0 = (m11 * g0 - m01 * g1) * idet, z1 = (m00 * g1 - m01 * g0) * idet;
             for (int r = 0; r < 3; ++r) {
-                const double cdd = z0 * e0[r] + z1 * e1[r];
-                const double ce0 = z0 * dv[r] - (z0 * (2.0 * s_ * e0[r] + t_ * e1[r]) + z1 * (s_ * e1[r]));
-                const double ce1 = z1 * dv[r] - (z0 * (t_ * e0[r]) + z1 * (s_ * e0[r] + 2.0 * t_ * e1[r]));
+                const double cdd = z0 * e1[r] + z1 * e2[r];
+                const double ce0 = z0 * P[r] - (z0 * (2.0 * s_ * e1[r] + t_ * e2[r]) + z1 * (s_ * e2[r]));
+                const double ce1 = z1 * P[r] - (z0 * (t_ * e1[r]) + z1 * (s_ * e1[r] + 2.0 * t_ * e2[r]));
                 acc[0][r] += -cdd - ce0 - ce1;
                 acc[1][r] += ce0;
                 acc[2][r] += ce1;
