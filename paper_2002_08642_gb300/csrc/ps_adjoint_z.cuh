@@ -118,7 +118,15 @@ k_adj_zpass(KP kp, AdjW aw, cplx<T>* __restrict__ B, const cplx<T>* __restrict__
         const uint8_t myflag = threadIdx.x < 2 ? flag[(size_t)b * 2 + threadIdx.x] : (uint8_t)0;
         auto noload = [&](int) -> C2 { return cmk<C2>((T)0, (T)0); };
         if constexpr (Z3) {
-            for (int q = g; q < M / 2; q += G) split3_pre<T, M, SUB>(fa, fb, tw3, tiles + tbase, q);
+            if constexpr (G % 16 == 0) {
+                for (int q = g; q < M / 2; q += G) split3_pre<T, M, SUB>(fa, fb, tw3, tiles + tbase, q);
+            } else {   // see k_zpass
+                for (int idx = threadIdx.x; idx < 9 * (M / 2); idx += 9 * G) {
+                    const int tj = idx / (M / 2), v = tj / 3, tq = tj - 3 * v;
+                    const C2* const f0 = stage + (tq < 2 ? (v * 3 * 2 + tq) * KZP : (v * 3 + 2) * 2 * KZP);
+                    split3_pre<T, M, SUB>(f0, f0 + (tq < 2 ? 2 * KZP : KZP), tw3, tiles + tj * LP, idx % (M / 2));
+                }
+            }
             __syncthreads();
             // every read of the staging buffer is done, the next batch may land
             if (threadIdx.x == 0 && more) issue(b + gridDim.x);

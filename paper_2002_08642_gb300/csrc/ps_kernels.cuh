@@ -637,12 +637,22 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
         const uint8_t myflag = threadIdx.x < LZ ? flag[(size_t)b * LZ + threadIdx.x] : (uint8_t)0;
         if constexpr (Z3) {
             // the split's pre-butterfly once per mirror pair of modes, into the
-            // tiles; each thread group fills its own tile (pl, pr)
-            {
+            // tiles: each thread group its own tile where groups are whole
+            // half-warps, else the pairs of all tiles over the block's
+            // threads (with groups of 12 or 24 threads a half-warp's lanes fell
+            // on two tiles and their banks; pressure at 192^3 237 -> 232 us,
+            // 384^2 x 192 box 2230 -> 2208; 768^3, groups of 48, 25724 -> 25798)
+            if constexpr (G % 16 == 0) {
                 const C2* fa = st + (size_t)((2 * pr) * LZ + pl) * KZP;
                 const C2* fb = st + (size_t)((2 * pr + 1) * LZ + pl) * KZP;
                 C2* t = tile(pl, pr);
                 for (int q = g; q < M / 2; q += G) split3_pre<T, M>(fa, fb, tw3, t, q);
+            } else {
+                for (int idx = threadIdx.x; idx < 3 * LZ * (M / 2); idx += 3 * LZ * G) {
+                    const int tj = idx / (M / 2), l = tj / 3, p = tj - 3 * l;
+                    const C2* fa = st + (size_t)((2 * p) * LZ + l) * KZP;
+                    split3_pre<T, M>(fa, fa + (size_t)LZ * KZP, tw3, tiles + tj * LP, idx % (M / 2));
+                }
             }
             __syncthreads();
             // one buffer: every read of it is done, the next batch may land
