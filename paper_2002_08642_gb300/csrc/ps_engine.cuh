@@ -5,9 +5,15 @@
 #include "ps_kernels.cuh"
 #include "ps_adjoint_z.cuh"
 
-// x-inverse: at most this many (ky, kz tile) tiles take the split kernel
+// x-inverse: at most this many (ky, kz tile) tiles take the split kernel. FP32:
+// fewer than two per SM of a GB300 (255 tiles, 128^3: plate run 705 -> 696 us;
+// 508 tiles, 192^3: pressure 237 -> 241). FP64, where the sixth transform
+// costs arithmetic: fewer than one (252 tiles, 96^3: step 489 -> 493 us)
 #ifndef PS_XSPLIT_TILES
-#define PS_XSPLIT_TILES 152
+#define PS_XSPLIT_TILES 256
+#endif
+#ifndef PS_XSPLIT_TILES_F64
+#define PS_XSPLIT_TILES_F64 152
 #endif
 
 namespace ps {
@@ -152,8 +158,9 @@ template <typename T, int N, int NZ = N> struct Engine {
         return g;
     }
     static constexpr int thr_x1 = GE::CX1 * GE::G;
-    // fewer (ky, kz tile) tiles than a GB300 has SMs: one item per output field
-    static constexpr bool XSPLIT = GE::K * (KZ_ / GE::CX1) <= PS_XSPLIT_TILES;
+    // too few (ky, kz tile) tiles to fill the SMs: one item per output field
+    static constexpr bool XSPLIT =
+        GE::K * (KZ_ / GE::CX1) <= (sizeof(T) == 8 ? PS_XSPLIT_TILES_F64 : PS_XSPLIT_TILES);
     // pass 1: x-inverse with the curl
     static void x_inverse(const KP& kp, const Bufs& b, cudaStream_t s) {
         const C2* tw = (const C2*)b.tw;
