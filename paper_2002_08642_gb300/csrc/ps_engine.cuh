@@ -151,7 +151,7 @@ template <typename T, int N, int NZ = N> struct Engine {
         return g;
     }
     static constexpr size_t sm_x1 = (size_t)GE::y2_smem(GE::CX1);
-    static constexpr size_t sm_x5t = (size_t)GE::x5_smem(GE::CX5);
+    static constexpr size_t sm_x5t = (size_t)XFwd<T, N, KZ_>::smem;
     static constexpr size_t sm_x5s = sm_x5t;   // the sponge variant keeps three result tiles
     static int& x5sgrid() {
         static int g = 0;
@@ -172,7 +172,7 @@ template <typename T, int N, int NZ = N> struct Engine {
             launch(k_xinv_tma<T, N, 6, KZ_>, x1grid(), thr_x1, sm_x1, s, *b.tmU, kp, (C2*)b.A, tw, b.err);
         }
     }
-    static constexpr int thr_x5 = GE::CX5 * GE::G;
+    static constexpr int thr_x5 = XFwd<T, N, KZ_>::threads;
     static constexpr size_t sm_y2 = (size_t)GE::y2_smem(GE::CY2, GE::Y2NB);
     static constexpr size_t sm_y4 = (size_t)GE::y4_smem(GE::CY4);
     static constexpr int thr_y2 = GE::CY2 * GE::G;

@@ -256,8 +256,9 @@ template <typename T, int N> struct Geo {
     static constexpr int y4_smem(int c) {   // y forward: 2 staging tiles of N rows, transformed in place
         return (int)sizeof(C2) * c * (2 * nbox(N) * bpitch(N, c)) + (int)sizeof(C2) * (tw_count(N, RM) + 1) + 256;
     }
-    static constexpr int x5_smem(int c, int nf = 3) {   // x forward: 2 staging tiles (N rows) + nf result tiles
-        return (int)sizeof(C2) * c * (2 * nbox(N) * bpitch(N, c) + nf * K) + (int)sizeof(C2) * (tw_count(N, RM) + 1) + 256;
+    // x forward: 2 staging buffers of grp fields (N rows each) + 3 result tiles
+    static constexpr int x5_smem(int c, int grp = 1) {
+        return (int)sizeof(C2) * c * (2 * grp * nbox(N) * bpitch(N, c) + 3 * K) + (int)sizeof(C2) * (tw_count(N, RM) + 1) + 256;
     }
     // widest tile (at most cmax complex, at least 2) whose shared memory fits
     static constexpr int pick_c(int which, int kb, int cmax) {
@@ -274,7 +275,13 @@ template <typename T, int N> struct Geo {
     static constexpr int CY2 = pick_c(2, PS_Y2_SMEM_KB, 16);
     static constexpr int CY4 = pick_c(4, PS_Y4_SMEM_KB, 16);
     static constexpr int CX1 = pick_c(1, PS_X1_SMEM_KB, 16);   // same smem shape as the y inverse, two buffers
-    static constexpr int CX5 = pick_c(5, PS_X5_SMEM_KB, 128 / 16);
+    // x forward: the widest tile; where there are fewer tiles than SMs,
+    // narrower as long as they have an SM each and are whole warps
+    static constexpr int x5_narrow(int c) {
+        while (c > 2 && 2 * K * (KZP / c) <= 152 && c / 2 * G % 32 == 0) c /= 2;
+        return c;
+    }
+    static constexpr int CX5 = x5_narrow(pick_c(5, PS_X5_SMEM_KB, 128 / 16));
     static constexpr int tw_n = tw_count(N, RM) > 0 ? tw_count(N, RM) : 1;
 };
 
@@ -1310,6 +1317,26 @@ k_xinv_split(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict_
     }
 }
 
+// x forward: fields in flight, each with a thread group and a staging buffer
+// of its own. One at a time, a tile is a chain of three transforms and a
+// projection by the same few warps; three at a time it is one transform and
+// a projection by three times as many.
+// FP32: where the three fields' buffers stay below 140 KB (n <= 256; 32^3 step
+// 15.4 -> 13.9 us, 48^3 19.0 -> 18.0, 128^3 59.6 -> 57.4, 192^3 185.4 -> 182.7,
+// 256^3 428.5 -> 425.2; at 384^2 x 192, 198 KB, the pass would take 159 us
+// instead of 155, at 512^3 and 768^3 with 4 columns 1043 instead of 959 and
+// 2315 instead of 1526). FP64 (a warp's instruction takes 64 cycles of a
+// quarter SM): where every warp has a quarter to itself (32^3 step 41.2 -> 32.9
+// us, 48^3 86.8 -> 82.3; 64^3 would go from 156.9 to 159.5).
+template <typename T, int N, int KZP_> struct XFwd {
+    using GE = Geo<T, N>;
+    static constexpr int TL = GE::CX5 * GE::G;   // threads of a transform
+    static constexpr int WARPS = GE::K * (KZP_ / GE::CX5) * 3 * ((TL + 31) / 32);
+    static constexpr bool FEW = sizeof(T) == 8 ? WARPS <= 4 * 152 : GE::x5_smem(GE::CX5, 3) <= 140 * 1024;
+    static constexpr int GRP = FEW && 3 * TL <= 1024 ? 3 : 1;
+    static constexpr int threads = GRP * TL, smem = GE::x5_smem(GE::CX5, GRP);
+};
+
 // pass 5 (TMA-staged): x-forward of the three fields of n, truncation to the
 // kept kx, 1/n^3, Leray projection and the integrating-factor AB2 (Euler on
 // the first step) update of U and H. MODE 1 instead sets U to the projected
@@ -1320,9 +1347,10 @@ k_xinv_split(const __grid_constant__ CUtensorMap tm, KP kp, cplx<T>* __restrict_
 // fields 0..2) + i k x (transform of fields 3..5), unscaled, and
 // mu <- -(dt/2) E^2 lam (0 for the Euler start step). Each field is
 // transformed in place in its staging buffer; kept outputs go to three result tiles.
+// GRP fields are in flight at a time (XFwd).
 // tm: A as rows of 2 Kzp reals, row (f K + ky) n + x.
 template <typename T, int N, int MODE, bool SP = false, int KZP_ = Geo<T, N>::KZP>
-__global__ void __launch_bounds__(Geo<T, N>::CX5 * Geo<T, N>::G)
+__global__ void __launch_bounds__(XFwd<T, N, KZP_>::threads)
 k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUtensorMap tmu,
            const __grid_constant__ CUtensorMap tmh, KP kp, cplx<T>* __restrict__ U, cplx<T>* __restrict__ H,
            const T* __restrict__ Ex, const T* __restrict__ Ez, int first, const cplx<T>* __restrict__ twg,
@@ -1336,7 +1364,8 @@ k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUten
     const int NTILE = kp.kyn * NTZ;   // tiles of this launch's ky rows
     constexpr uint32_t box_bytes = (uint32_t)(BR * CT * sizeof(C2));
     extern __shared__ __align__(16) unsigned char smraw[];
-    C2* S = reinterpret_cast<C2*>(smem_base128(smraw));   // [2][RS][CT]
+    constexpr int GRP = XFwd<T, N, KZP_>::GRP, TL = XFwd<T, N, KZP_>::TL;
+    C2* S = reinterpret_cast<C2*>(smem_base128(smraw));   // [2][GRP][RS][CT]
     if (smem_u32(S) & 127u) {
         pdl_wait();
         if (threadIdx.x == 0) atomicExch(err, 2);
@@ -1344,12 +1373,13 @@ k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUten
     }
     // fields read: n (A fields 0..2), with the sponge first s (A fields 3..5),
     // whose sponge term -(1/C_sp) i k x s_hat/|k|^2 the n transforms add onto
-    constexpr int NF = SP ? 6 : 3;
+    constexpr int NF = SP ? 6 : 3, NR = NF / GRP;   // fields, rounds of GRP fields
     auto field = [](int j) { return SP ? (j < 3 ? j + 3 : j - 3) : j; };
-    C2* Rt = S + 2 * RS * CT;                             // [3][K][CT]
+    C2* Rt = S + 2 * GRP * RS * CT;                       // [3][K][CT]
     C2* tw = Rt + 3 * K * CT;
     __shared__ __align__(8) uint64_t bar[2];
-    const int col = threadIdx.x % CT, g = threadIdx.x / CT;
+    const int gi = threadIdx.x / TL, tl = threadIdx.x % TL;   // the round's field of this thread
+    const int col = tl % CT, g = tl / CT;
     const int mmax = kp.mmax, Kz = kp.Kz;
     const size_t FS = (size_t)K * K * KZP;
     if (threadIdx.x == 0) {
@@ -1362,13 +1392,15 @@ k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUten
     __syncthreads();
     pdl_wait();
     auto issue = [&](int L) {  // one thread
-        const int t = blockIdx.x + (L / NF) * gridDim.x, f = field(L % NF), buf = L & 1;
+        const int t = blockIdx.x + (L / NR) * gridDim.x, buf = L & 1;
         if (t >= NTILE) return;
         const int cy = kp.ky0 + t / NTZ, czt = t % NTZ;
         fence_proxy_async();
-        mbar_arrive_expect_tx(&bar[buf], NBOX * box_bytes);
-        for (int b = 0; b < NBOX; ++b)
-            tma_load_2d(S + (size_t)(buf * RS + b * BP) * CT, &tm, 2 * czt * CT, (f * K + cy) * N + b * BR, &bar[buf]);
+        mbar_arrive_expect_tx(&bar[buf], GRP * NBOX * box_bytes);
+        for (int i = 0; i < GRP; ++i)
+            for (int b = 0; b < NBOX; ++b)
+                tma_load_2d(S + (size_t)((buf * GRP + i) * RS + b * BP) * CT, &tm, 2 * czt * CT,
+                            (field(L % NR * GRP + i) * K + cy) * N + b * BR, &bar[buf]);
     };
     if (threadIdx.x == 0) issue(0);
     const T s = (T)kp.ks, sz = (T)kp.ksz;
@@ -1387,9 +1419,9 @@ k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUten
             tma_prefetch_2d(MODE == 3 || first ? &tmu : &tmh, 2 * czt * CT, (f * K + cy) * K + b * BRK);
         }
 #pragma unroll 1
-        for (int j = 0; j < NF; ++j) {
-            const int L = NF * ti + j, buf = L & 1, f = field(j) % 3;
-            const bool acc = SP && j >= 3;   // n onto the sponge term
+        for (int j = 0; j < NR; ++j) {
+            const int L = NR * ti + j, buf = L & 1, f = field(j * GRP + gi) % 3;
+            const bool acc = SP && j * GRP >= 3;   // n onto the sponge term
             if (threadIdx.x == 0) issue(L + 1);
             const bool ok = mbar_wait(&bar[buf], (uint32_t)((L >> 1) & 1));
             if (__syncthreads_or(!ok)) {
@@ -1400,7 +1432,7 @@ k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUten
                 stop = true;
                 break;
             }
-            C2* Sb = S + (size_t)buf * RS * CT;
+            C2* Sb = S + (size_t)(buf * GRP + gi) * RS * CT;
             C2* Rf = Rt + f * K * CT;
             auto noload = [&](int) -> C2 { return cmk<C2>((T)0, (T)0); };
             if constexpr (S3::on) {
@@ -1412,7 +1444,7 @@ k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUten
                 auto store = [&](int p, C2 v) { S[addr3(p)] = v; };
                 S3::template FFT<-1>::template run<true>(S, tw, addr3, gm, noload, store);
                 __syncthreads();
-                for (int idx = threadIdx.x; idx < M * CT; idx += blockDim.x) {
+                for (int idx = tl; idx < M * CT; idx += TL) {
                     const int kq = idx / CT, c = idx % CT;
                     C2 Zk, Zm;
                     split3_out(Sb[(3 * kq) * CT + c], Sb[(3 * kq + 1) * CT + c], Sb[(3 * kq + 2) * CT + c], tw3, kq,
@@ -1437,7 +1469,7 @@ k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUten
             }
             __syncthreads();
             if constexpr (SP) {
-                if (j == 2) {   // s_hat complete: replace it by the sponge term (MODE 3: by i k x s_hat)
+                if (j == 3 / GRP - 1) {   // s_hat complete: replace it by the sponge term (MODE 3: by i k x s_hat)
                     const T myy = (T)cmode_of(cy, mmax, K);
                     for (int idx = threadIdx.x; idx < K * CT; idx += blockDim.x) {
                         const int cx = idx / CT, czz = czt * CT + idx % CT;
@@ -1485,7 +1517,7 @@ k_xfwd_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ CUten
             nn[0] = n0; nn[1] = n1; nn[2] = n2;
         };
         // points per thread: every load of a point issued before its arithmetic
-        constexpr int NT = CT * G, NPT = (K * CT + NT - 1) / NT;
+        constexpr int NT = GRP * TL, NPT = (K * CT + NT - 1) / NT;
 #pragma unroll
         for (int r = 0; r < NPT; ++r) {
             const int idx = threadIdx.x + r * NT;
