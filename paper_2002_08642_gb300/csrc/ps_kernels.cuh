@@ -648,8 +648,9 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
             // half-warps, else the pairs of all tiles over the block's
             // threads (with groups of 12 or 24 threads a half-warp's lanes fell
             // on two tiles and their banks; pressure at 192^3 237 -> 232 us,
-            // 384^2 x 192 box 2230 -> 2208; 768^3, groups of 48, 25724 -> 25798)
-            if constexpr (G % 16 == 0) {
+            // 384^2 x 192 box 2230 -> 2208; 768^3, groups of 48, 25724 -> 25798;
+            // FP64, bound by arithmetic, 192^3 step 4190 -> 4230)
+            if constexpr (sizeof(T) == 8 || G % 16 == 0) {
                 const C2* fa = st + (size_t)((2 * pr) * LZ + pl) * KZP;
                 const C2* fb = st + (size_t)((2 * pr + 1) * LZ + pl) * KZP;
                 C2* t = tile(pl, pr);
@@ -696,6 +697,10 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
         __syncthreads();
         // one buffer: every read of it is done, the next batch may land
         if (!Z3 && NB == 1 && threadIdx.x == 0 && more) issue(b + gridDim.x, 0);
+        // lines whose pass gains from the flagged lines' loads ahead of their
+        // use and from forward transforms in the first groups: see there
+        constexpr bool SHORT = sizeof(T) == 8 ? N <= 128 : Z3 || G <= 16;
+        constexpr bool EAGER = SHORT || G <= 16;
         using Sum = typename sum_of<T>::type;
         Sum fm[6] = {};   // q and (offset from jc in cells) x q
         bool touched = false;
@@ -710,10 +715,11 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
             nz = ux * wy - uy * wx;
             if constexpr (PM) half_u2[(size_t)lid * N + z] = (T)0.5 * (ux * ux + uy * uy + uz * uz);
             if (sflag[l] != 0) {
-                const T c = cs[0];
+                const size_t po = (size_t)lid * N + z;
+                const T c = EAGER ? cs[0] : chi[po];
                 if (c != (T)0) {
                     const int x = (int)(lid / nyl), y = (int)(lid % nyl);
-                    const T sx = cs[1], sy = cs[2], sz = cs[3];
+                    const T sx = EAGER ? cs[1] : us[po], sy = EAGER ? cs[2] : us[N3 + po], sz = EAGER ? cs[3] : us[2 * N3 + po];
                     const T ce = c * inv_eta;
                     nx -= ce * (ux - sx);
                     ny -= ce * (uy - sy);
@@ -747,11 +753,14 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
             // once (one memory latency per round, also where chi turns out 0;
             // loading u_s after chi, line after line, took four; with the
             // register budget of short lines: plate 128^3 805 -> 758 us,
-            // wing 256^3 2164 -> 2136)
+            // wing 256^3 2164 -> 2136). Not EAGER: inside nonlinear; FP32 lines of
+            // 512 points and long FP64 lines, where the registers cost more, also
+            // with no mask (step at 512^3 3713 -> 3662 us, 768^3 FP64 270.3 -> 269.2
+            // ms; the FP32 768^3 wing the other way, 25804 -> 25927 us)
             T cs[2][4];
 #pragma unroll
             for (int j = 0; j < 2; ++j)
-                if (sflag[l + j] != 0) {
+                if (EAGER && sflag[l + j] != 0) {
                     const size_t po = ((size_t)b * LZ + l + j) * N + z;
                     cs[j][0] = chi[po];
                     cs[j][1] = us[po];
@@ -805,12 +814,16 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
         }
         __syncthreads();
         {
-            // forward lines: (l, 0) for every l, (l, 1) for even l, by the
-            // first groups; the rest (whole warps of them) idle. With the
-            // sponge every tile
-            constexpr int NJ = SP ? 3 * LZ : LZ + LZ / 2;
-            const bool active = fl < NJ;
-            const int jl = SP ? pl : fl < LZ ? fl : active ? 2 * (fl - LZ) : 0, jp = SP ? pr : fl < LZ ? 0 : 1;
+            // forward lines: (l, 0) for every l, (l, 1) for even l; FIRST: by
+            // the first groups, so that the rest idle as whole warps (step at
+            // 384^3 1339 -> 1313 us, 768^3 10801 -> 10770, 96^3 FP64 507 -> 465), else
+            // by the tiles' own groups (512^3 3704 -> 3662 us, FP64 192^3 4190 ->
+            // 4104, 768^3 273.3 -> 270.3 ms). With the sponge every tile
+            constexpr int NJ = LZ + LZ / 2;
+            constexpr bool FIRST = !SP && SHORT;
+            const bool active = SP || (FIRST ? fl < NJ : pr == 0 || (pr == 1 && (pl & 1) == 0));
+            const int jl = !FIRST || fl < LZ ? (FIRST ? fl : pl) : active ? 2 * (fl - LZ) : 0;
+            const int jp = FIRST ? (fl < LZ ? 0 : 1) : SP || pr < 2 ? pr : 1;
             const int tbase = (int)(tile(jl, jp) - tiles);
             auto noload = [&](int) -> C2 { return cmk<C2>((T)0, (T)0); };
             if constexpr (Z3) {
