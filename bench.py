@@ -79,10 +79,9 @@ def algorithmic_bytes(n, elem_complex, flagged_lines=0, elem_real=4, nz=None):
 
 
 def adjoint_bytes(n, elem_complex, elem_real):
-    """Algorithmic bytes of one reversed step (ps_adjoint_step, FP32 or
-    FP64 storage), per kernel family; the checkpoint recompute of the
-    forward steps and the rasteriser VJP (band points only) are not counted.
-    State arrays are 3 x K^2 Kz (lam, mu, G, Ub, Wb), z-spectral 3 x n^2 Kz,
+    """Bytes of one reversed step if its z transforms, pointwise term and
+    spectral updates were separate kernels (FP32 or FP64 storage), per kernel
+    family; ps_adjoint_step moves fewer (adjoint_fused_bytes). State arrays are 3 x K^2 Kz (lam, mu, G, Ub, Wb), z-spectral 3 x n^2 Kz,
     physical 3 x n^3."""
     mm = (n - 1) // 3
     K, Kz = 2 * mm + 1, mm + 1
@@ -96,6 +95,23 @@ def adjoint_bytes(n, elem_complex, elem_real):
         "pointwise": 23 * n3 * r_,                                   # u, w, nbar, chi, u_s in; ubar, wbar, grads out
         "forward_2x3": 2 * (3 * n3 * r_ + 3 * nn * e + (3 * nn + 3 * nk) * e + (3 * nk + 3 * kk) * e),
         "spectral_2": 12 * kk * e,                                   # lam, Ub, Wb in; lam out
+    }
+
+
+def adjoint_fused_bytes(n, elem_complex, elem_real):
+    """Algorithmic bytes of one reversed step (ps_adjoint_step, FP32 or FP64
+    storage), per kernel family; the checkpoint recompute of the forward
+    steps and the rasteriser VJP (band points only) are not counted."""
+    mm = (n - 1) // 3
+    K, Kz = 2 * mm + 1, mm + 1
+    kk, nk, nn = K * K * Kz, n * K * Kz, n * n * Kz
+    e, r_ = elem_complex, elem_real
+    return {
+        "spectral": 9 * kk * e,                                      # lam, mu in; G out
+        "inverse_u_omega": (3 * kk + 6 * nk) * e + (6 * nk + 6 * nn) * e,
+        "inverse_G": (3 * kk + 3 * nk) * e + (3 * nk + 3 * nn) * e,
+        "z_fused": 15 * nn * e + 8 * n ** 3 * r_,                    # u, w, nbar in; ubar, wbar out; chi, u_s, grads
+        "forward": (6 * nn + 6 * nk) * e + (6 * nk + 9 * kk) * e,    # lam in; lam, mu out
     }
 
 
@@ -453,9 +469,9 @@ def run_ours(args, cfg):
     peak, src = peaks()
     achieved = ab[top] / (tms / tl / 1e3) / 1e9
     step_bytes = sum(ab.values())
-    # five passes + rasteriser (clear with node positions, triangle boxes,
-    # prefix sum, pair pass, evaluate; FP64 adds a second pair pass)
-    kernels_per_step = 5 + (5 if cfg["precision"] == "fp32" else 6)
+    # five passes + rasteriser (clear with node positions and triangle boxes,
+    # pair walk, evaluate; FP64 walks the pairs three times)
+    kernels_per_step = 5 + (3 if cfg["precision"] == "fp32" else 5)
     # the z pass against the FP32 FMA rate: its line transforms (4.5 complex
     # length-n transforms per (x, y) line, 5 n log2 n FLOPs each) and the
     # pointwise term; it is bound by instruction issue, not by FMA throughput
@@ -625,13 +641,14 @@ def run_ours(args, cfg):
         e1.record(stream)
         torch.cuda.synchronize()
         msa = e0.elapsed_time(e1)
-        adj_b = adjoint_bytes(na, 8, 4)
+        adj_b = adjoint_fused_bytes(na, 8, 4)
         pk, src_ = peaks()
         adj_tot = sum(adj_b.values())
         out["adjoint_step"] = {"value": na ** 3 * ka / (msa / 1e3) / 1e6, "unit": "Mpts*steps/s", "n": na,
                                "precision": "fp32", "steps": ka, "ms_per_step": msa / ka,
                                "roofline": {"bound": "hbm", "algorithmic_bytes_per_step": adj_tot,
                                             "bytes_by_kernel_family": adj_b,
+                                            "unfused_bytes_per_step": sum(adjoint_bytes(na, 8, 4).values()),
                                             "achieved": adj_tot / (msa / ka / 1e3) / 1e9, "peak": pk,
                                             "unit": "GB/s", "frac": adj_tot / (msa / ka / 1e3) / 1e9 / pk,
                                             "peak_source": src_},
