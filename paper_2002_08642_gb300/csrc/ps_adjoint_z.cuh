@@ -118,7 +118,7 @@ k_adj_zpass(KP kp, AdjW aw, cplx<T>* __restrict__ B, const cplx<T>* __restrict__
         const uint8_t myflag = threadIdx.x < 2 ? flag[(size_t)b * 2 + threadIdx.x] : (uint8_t)0;
         auto noload = [&](int) -> C2 { return cmk<C2>((T)0, (T)0); };
         if constexpr (Z3) {
-            if constexpr (sizeof(T) == 8 || G % 16 == 0) {
+            if constexpr (G % 16 == 0 || (sizeof(T) == 8 && N > 128)) {
                 for (int q = g; q < M / 2; q += G) split3_pre<T, M, SUB>(fa, fb, tw3, tiles + tbase, q);
             } else {   // see k_zpass
                 for (int idx = threadIdx.x; idx < 9 * (M / 2); idx += 9 * G) {

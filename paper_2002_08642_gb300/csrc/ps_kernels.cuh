@@ -649,8 +649,8 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
             // threads (with groups of 12 or 24 threads a half-warp's lanes fell
             // on two tiles and their banks; pressure at 192^3 237 -> 232 us,
             // 384^2 x 192 box 2230 -> 2208; 768^3, groups of 48, 25724 -> 25798;
-            // FP64, bound by arithmetic, 192^3 step 4190 -> 4230)
-            if constexpr (sizeof(T) == 8 || G % 16 == 0) {
+            // FP64 96^3 step 490 -> 465, but 192^3 4190 -> 4230)
+            if constexpr (G % 16 == 0 || (sizeof(T) == 8 && N > 128)) {
                 const C2* fa = st + (size_t)((2 * pr) * LZ + pl) * KZP;
                 const C2* fb = st + (size_t)((2 * pr + 1) * LZ + pl) * KZP;
                 C2* t = tile(pl, pr);
