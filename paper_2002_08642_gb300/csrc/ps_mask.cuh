@@ -77,7 +77,7 @@ static constexpr int kMaskMaxNodes = 1 << 17;
 // their dot products; the lengths rounded once from double to T. A grid point
 // minus a is then (i - ca) dx - f, with no double arithmetic per pair.
 // m, r: a sphere around the triangle (centre relative to a); nrm: the unit
-// normal (0 for a degenerate triangle).
+// normal, 0 for a triangle without a plane (has_plane; such a one gives no bounds).
 template <typename T> struct TriGeo {
     int i0[3], e[3], ca[3];
     float r;
@@ -178,11 +178,14 @@ __device__ __forceinline__ bool le0(float x) { return x <= 0.0f; }
 __device__ __forceinline__ bool ge0(float x) { return x >= 0.0f; }
 __device__ __forceinline__ bool le0(double x) { return __double_as_longlong(x) <= 0; }
 __device__ __forceinline__ bool ge0(double x) { return __double2hiint(x) >= 0; }
+__device__ __forceinline__ bool is0(float x) { return x == 0.0f; }
+__device__ __forceinline__ bool is0(double x) { return (__double_as_longlong(x) << 1) == 0; }
 
 // Barycentrics (v of b, w of c) of the point of the triangle (0, b, c) closest
 // to P, by the same region tests as closest_tri with the dot products
 // relative to vertex a: bp = P - b and cp = P - c enter through
-// ab . bp = ab . P - ab . ab and so on.
+// ab . bp = ab . P - ab . ab and so on. Vertices at one place (the chosen
+// region's denominator is 0): the closest point of the longer of ab and ac.
 template <typename R>
 __device__ __forceinline__ void closest_rel(const R P[3], const R b[3], const R c[3], R bb, R bc, R cc, R& v, R& w) {
     const R d1 = b[0] * P[0] + b[1] * P[1] + b[2] * P[2];
@@ -198,13 +201,35 @@ __device__ __forceinline__ void closest_rel(const R P[3], const R b[3], const R 
     // one division for all remaining regions: an edge's or the face's parameter
     const bool e_ab = le0(vc) && ge0(d1) && le0(d3);
     const bool e_ac = !e_ab && le0(vb) && ge0(d2) && le0(d6);
-    const bool e_bc = !e_ab && !e_ac && le0(va) && ge0(d43) && ge0(d56);
-    const R den = e_ab ? d1 - d3 : e_ac ? d2 - d6 : e_bc ? d43 + d56 : va + vb + vc;
+    const R l_bc = d43 + d56;   // |c - b|^2; 0: va is rounding
+    const bool e_bc = !e_ab && !e_ac && (le0(va) || le0(l_bc)) && ge0(d43) && ge0(d56);
+    const R den = e_ab ? d1 - d3 : e_ac ? d2 - d6 : e_bc ? l_bc : va + vb + vc;
+    if (is0(den)) {
+        const bool ac = cc >= bb;
+        const R len = ac ? cc : bb;
+        const R p = len > (R)0 ? fmin(fmax((ac ? d2 : d1) / len, (R)0), (R)1) : (R)0;
+        v = ac ? (R)0 : p;
+        w = ac ? p : (R)0;
+        return;
+    }
     const R q = (R)1 / den;
     if (e_ab) { v = d1 * q; w = 0; }
     else if (e_ac) { v = 0; w = d2 * q; }
     else if (e_bc) { w = d43 * q; v = (R)1 - w; }
     else { v = vb * q; w = vc * q; }
+}
+
+// Whether the FP32 bounds of the FP64 walks hold for a triangle: big the
+// largest component of its edges' cross product, l2 its longest edge squared,
+// len the size of the coordinates. They take the triangle to lie in the plane of
+// its normal, and the exact test to find its distance to 1e-5 of len. Both need
+// an area: with the rounding of nearly parallel edges (or coincident vertices,
+// 0 / 0) the normal points anywhere and the exact test's weights are rounding
+// too, or no numbers. A height of at least 1/1000 of the longest edge leaves
+// the exact test an error of 1e-10 len^2 / edge. FP32 squares of the
+// coordinates must not leave the range either. No comparison holds for a NaN.
+__device__ __forceinline__ bool has_plane(float big, float l2, float len) {
+    return big >= 6e-4f * l2 && l2 > 1e-30f && len > 1e-15f && len < 1e15f;
 }
 
 // Box and pair-test geometry of triangle t, axis r = 0..2 by lanes 4 q + r of
@@ -280,11 +305,18 @@ __device__ __forceinline__ void tri_setup(const MaskWs& m, const MaskArgs& a, in
         if constexpr (sizeof(T) == 8) {   // unit normal (only the FP64 walks use it)
             const float n[3] = {(float)(vb[1] * vc[2] - vb[2] * vc[1]), (float)(vb[2] * vc[0] - vb[0] * vc[2]),
                                 (float)(vb[0] * vc[1] - vb[1] * vc[0])};
-            // scaled by the largest component: no underflow of tiny areas' squares
+            float l2 = 0.0f, bb = 0.0f, cc = 0.0f;   // squared edge lengths
+            for (int q = 0; q < 3; ++q) {
+                const float fb = (float)vb[q], fc = (float)vc[q];
+                bb += fb * fb;
+                cc += fc * fc;
+                l2 += (fb - fc) * (fb - fc);
+            }
+            l2 = fmaxf(l2, fmaxf(bb, cc));
             const float big = fmaxf(fabsf(n[0]), fmaxf(fabsf(n[1]), fabsf(n[2])));
-            const float k = big > 0.0f ? 1.0f / big : 0.0f;
-            const float x = n[0] * k, y = n[1] * k, z = n[2] * k, len = x * x + y * y + z * z;
-            const float u = len >= 0.5f ? rsqrtf(len) : 0.0f;   // 0: degenerate (no area)
+            const bool plane = has_plane(big, l2, sqrtf(l2) + (float)(reach + a.dx));
+            const float k = plane ? 1.0f / big : 0.0f;
+            const float x = n[0] * k, y = n[1] * k, z = n[2] * k, u = plane ? rsqrtf(x * x + y * y + z * z) : 0.0f;
             g.nrm[0] = x * u;
             g.nrm[1] = y * u;
             g.nrm[2] = z * u;
@@ -401,11 +433,14 @@ __global__ void __launch_bounds__(kPairThreads) k_mask_pairs(MaskWs m, MaskArgs 
         }
     } else {
         // FP32 bounds of a pair's distance: the triangle lies in the disc of
-        // radius r about m in its plane (a ball if it has no normal), and a
-        // point of it with clamped barycentrics is at least as far as the
-        // closest one. Both are rounded outwards by err, ten times the
-        // rounding of coordinates of this size.
-        const float fdx = (float)a.dx, freach = (float)reach, err = 1e-5f * (g.r + freach);
+        // radius r about m in its plane, and a point of it with clamped
+        // barycentrics is at least as far as the closest one. Both are
+        // rounded outwards by err, some thirty times the rounding of the
+        // coordinates (at most 2 r + reach + a cell, 1.2e-7 of that). A
+        // triangle without a plane bounds nothing: its points go to the list
+        // with an infinite key and every pair of its box to the exact test.
+        const bool plane = g.nrm[0] != 0.0f || g.nrm[1] != 0.0f || g.nrm[2] != 0.0f;
+        const float fdx = (float)a.dx, freach = (float)reach, err = 1e-5f * (g.r + freach + fdx);
         const float ff[3] = {(float)g.f[0], (float)g.f[1], (float)g.f[2]};
         auto at = [&](int i, int j, int k, float* P) {
             P[0] = (float)(i - g.ca[0]) * fdx - ff[0];
@@ -413,6 +448,7 @@ __global__ void __launch_bounds__(kPairThreads) k_mask_pairs(MaskWs m, MaskArgs 
             P[2] = (float)(k - g.ca[2]) * fdx - ff[2];
         };
         auto lower = [&](const float* P) {
+            if (!plane) return 0.0f;
             const float x = P[0] - g.m[0], y = P[1] - g.m[1], z = P[2] - g.m[2];
             const float h = x * g.nrm[0] + y * g.nrm[1] + z * g.nrm[2], h2 = h * h;
             const float in = fmaxf(sqrtf(fmaxf(x * x + y * y + z * z - h2, 0.0f)) - g.r - err, 0.0f);
@@ -426,6 +462,10 @@ __global__ void __launch_bounds__(kPairThreads) k_mask_pairs(MaskWs m, MaskArgs 
                 float P[3], v, w, s = 0.0f;
                 at(i, j, k, P);
                 if (lower(P) > freach) continue;
+                if (!plane) {
+                    offer(index(i, j, k), 0x7ff0000000000000ull);
+                    continue;
+                }
                 closest_rel<float>(P, b, c, (float)g.bb, (float)g.bc, (float)g.cc, v, w);
                 v = fminf(fmaxf(v, 0.0f), 1.0f);
                 w = fminf(fmaxf(w, 0.0f), 1.0f - v);
