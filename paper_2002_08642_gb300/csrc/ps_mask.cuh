@@ -178,6 +178,7 @@ __device__ __forceinline__ bool le0(float x) { return x <= 0.0f; }
 __device__ __forceinline__ bool ge0(float x) { return x >= 0.0f; }
 __device__ __forceinline__ bool le0(double x) { return __double_as_longlong(x) <= 0; }
 __device__ __forceinline__ bool ge0(double x) { return __double2hiint(x) >= 0; }
+__device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 __device__ __forceinline__ bool is0(float x) { return x == 0.0f; }
 __device__ __forceinline__ bool is0(double x) { return (__double_as_longlong(x) << 1) == 0; }
 
@@ -269,7 +270,9 @@ __device__ __forceinline__ void tri_setup(const MaskWs& m, const MaskArgs& a, in
     TriGeo<T>& g = *reinterpret_cast<TriGeo<T>*>(m.geo + (size_t)t * kTriGeoBytes);
     int i0 = 0, e = 0, ca = 0;
     T f = (T)0;
-    if (good) {
+    // a vertex that is no number has no box, so no pair (fmin and fmax would
+    // leave it out, and with all three the box would be the whole grid)
+    if (good && finite(X[0]) && finite(X[1]) && finite(X[2])) {
         double l = ceil((fmin(X[0], fmin(X[1], X[2])) - reach) * a.inv_dx);
         double h = floor((fmax(X[0], fmax(X[1], X[2])) + reach) * a.inv_dx);
         l = fmax(l, ax == 0 ? (double)a.x_lo : 0.0);
