@@ -108,6 +108,8 @@ bool layout_for(const ps_params* p, const Ops* ops, Layout* L) {
     L->tw = take((size_t)3 * (n + nz) * ec);
     L->Ex = take((size_t)K * er);
     L->Ez = take((size_t)Kz * er);
+    // six sums per block of the z pass (at most a block per line), then room
+    // for the diagnostics' partial sums
     const size_t nparts = (size_t)n * n + 4096;
     L->partial = take(nparts * 6 * sizeof(double));
     L->out = take(64 * sizeof(double));
@@ -933,9 +935,10 @@ ps_status ps_diagnostics(ps_ctx* c, double* energy, double* max_div) {
     if (!energy || !max_div) return fail(c, PS_EINVAL, "ps_diagnostics: null output");
     DeviceGuard dg(c->device);
     const int nb = 304;
-    if (c->fp64) launch(k_diag<double>, nb, 256, 0, c->stream, c->kp, (const double2*)c->b.U, c->b.partial);
-    else launch(k_diag<float>, nb, 256, 0, c->stream, c->kp, (const float2*)c->b.U, c->b.partial);
-    launch(k_diag_final, 1, 32, 0, c->stream, c->b.partial, nb, c->kp.half_L3, c->out + 8);
+    double* const part = c->b.partial + (size_t)c->p.n * c->p.n * 6;   // behind the z pass's slots, which ps_forces reads
+    if (c->fp64) launch(k_diag<double>, nb, 256, 0, c->stream, c->kp, (const double2*)c->b.U, part);
+    else launch(k_diag<float>, nb, 256, 0, c->stream, c->kp, (const float2*)c->b.U, part);
+    launch(k_diag_final, 1, 32, 0, c->stream, part, nb, c->kp.half_L3, c->out + 8);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(c, e, "ps_diagnostics");
     double h[3];
