@@ -69,7 +69,10 @@ enum { PS_MEAN_FIXED = 0, PS_MEAN_FREE = 1 };
  *              and the 2/3 rule keeps 3|m_z| < nz. Other values return
  *              PS_EUNSUPPORTED.
  *   precision  PS_FP32: transforms, nonlinear term, projection and update in
- *              float, force/moment/diagnostic reductions in double;
+ *              float, diagnostic reductions in double, force/moment sums
+ *              at least as exact as sums in double (a point's and a warp's
+ *              terms chi (u - u_s) in three floats each, which keeps float's
+ *              exponent range; doubles from there on);
  *              PS_FP64: everything in double.
  *   mask_profile  profile used by ps_set_mask_from_nodes: PS_MASK_COS is
  *              Sec. 4.1 Eq. (mask_function) (banded, chi = 0 beyond t_w + h);

@@ -32,7 +32,7 @@
 //   1 x-inverse of u_hat and omega_hat = i k x u_hat (curl fused)    U -> A (6)
 //   2 y-inverse                                                      A -> B (6)
 //   3 z c2r, n = u x omega - (chi/eta)(u - u_s), force/moment partial
-//     sums in double, z r2c truncated to Kz                          B -> B (3)
+//     sums as exact as doubles (sum_of), z r2c truncated to Kz       B -> B (3)
 //   4 y-forward truncated to K rows                                  B -> A (3)
 //   5 x-forward truncated to K rows, 1/n^3, P, integrating-factor
 //     AB2 (Euler on the first step)                                  A,U,H -> U,H
@@ -125,46 +125,74 @@ struct Acc {
 
 // Penalization sums of the z pass: q = chi (u - u_s) of a point and a thread's
 // running sums of q and of whole-cell offsets times q. FP64 fields: doubles.
-// FP32 fields: unevaluated FP32 pairs (h + l, about 48 bits: exact difference
-// and product by two-sum and fused multiply-add, the rounding of l is the
-// error), summed over the few points a thread has in a batch and over its
-// warp, then added to the compensated doubles. An FP64 instruction takes 64
-// cycles of a quarter SM, an FP32 one a cycle: with the sums in doubles from
-// the point on, 31 FP64 instructions per masked point and 66 per warp made up
-// most of the pass where the mask fills many lines (GB300: static plate at
-// 128^3 83 -> 42 us per pass, wing at 48^3 17 -> 11 us, at 256^3 173 -> 164).
-struct Pair32 {
-    float h, l;
+// FP32 fields: unevaluated sums of three FP32 words (h + m + l, 72 bits; exact
+// differences, sums and products by two-sum and fused multiply-add, only l is
+// rounded), summed over the few points a thread has in a batch and over its
+// warp, then rounded once to the compensated doubles: no further from the
+// sum of the same q in 64 bits than doubles from the point on (two words, 48
+// bits, would be). The words have FP32's exponents: what lies below 1e-45 is
+// lost, and q times its offset must stay below 3.4e38.
+// An FP64 instruction takes 64 cycles of a quarter SM, an FP32 one a cycle:
+// with the sums in doubles from the point on, 31 FP64 instructions per masked
+// point and 66 per warp made up most of the pass where the mask fills many
+// lines (GB300, static plate at 128^3: 83 us per pass against 42 with two words
+// when that was changed; as the pass is now 33.2 us with two words, 35.0 with
+// three; wing at 48^3 12.4 and 12.6, at 256^3 161 and 159).
+struct Tri32 {
+    float h, m, l;
 };
-__device__ __forceinline__ Pair32 pair_sum(float a, float b) {   // a + b exactly
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {   // a + b = sum + e
     const float s = __fadd_rn(a, b), t = __fadd_rn(s, -a);
-    return {s, __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -t)), __fadd_rn(b, -t))};
+    e = __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -t)), __fadd_rn(b, -t));
+    return s;
 }
-__device__ __forceinline__ Pair32 pair_mul(float j, Pair32 q) {
-    const float h = __fmul_rn(j, q.h);
-    return {h, __fmaf_rn(j, q.l, __fmaf_rn(j, q.h, -h))};
+__device__ __forceinline__ void sum_add(Tri32& a, Tri32 q) {
+    float e, f, g;
+    a.h = two_sum(a.h, q.h, e);
+    a.m = two_sum(two_sum(a.m, q.m, f), e, g);
+    a.l = __fadd_rn(a.l, __fadd_rn(__fadd_rn(f, g), q.l));
 }
-__device__ __forceinline__ void sum_add(Pair32& a, Pair32 q) {
-    const Pair32 s = pair_sum(a.h, q.h);
-    a.h = s.h;
-    a.l = __fadd_rn(a.l, __fadd_rn(s.l, q.l));
+__device__ __forceinline__ Tri32 tri_mul(float j, Tri32 q) {
+    Tri32 r;
+    float e;
+    r.h = __fmul_rn(j, q.h);
+    const float m = __fmul_rn(j, q.m);
+    r.m = two_sum(m, __fmaf_rn(j, q.h, -r.h), e);
+    r.l = __fadd_rn(__fmaf_rn(j, q.l, __fmaf_rn(j, q.m, -m)), e);
+    return r;
 }
+__device__ __forceinline__ Tri32 neg(Tri32 q) { return {-q.h, -q.m, -q.l}; }
 __device__ __forceinline__ void sum_add(double& a, double q) { a += q; }
-__device__ __forceinline__ void sum_fma(Pair32& a, float j, Pair32 q) { sum_add(a, pair_mul(j, q)); }
+__device__ __forceinline__ void sum_fma(Tri32& a, float j, Tri32 q) { sum_add(a, tri_mul(j, q)); }
 __device__ __forceinline__ void sum_fma(double& a, double j, double q) { a = fma(j, q, a); }
-__device__ __forceinline__ Pair32 pen_term(float c, float u, float s) { return pair_mul(c, pair_sum(u, -s)); }
+__device__ __forceinline__ Tri32 pen_term(float c, float u, float s) {
+    Tri32 r;
+    float e, f;
+    const float d = two_sum(u, -s, e), m = __fmul_rn(c, e);
+    r.h = __fmul_rn(c, d);
+    r.m = two_sum(m, __fmaf_rn(c, d, -r.h), f);
+    r.l = __fadd_rn(__fmaf_rn(c, e, -m), f);
+    return r;
+}
 __device__ __forceinline__ double pen_term(double c, double u, double s) { return c * (u - s); }
-__device__ __forceinline__ double sum_val(Pair32 a) { return (double)a.h + (double)a.l; }
+__device__ __forceinline__ double sum_val(Tri32 a) { return (double)a.h + ((double)a.m + (double)a.l); }
 __device__ __forceinline__ double sum_val(double a) { return a; }
-__device__ __forceinline__ Pair32 sum_down(unsigned m, Pair32 a, int o) {
-    return {__shfl_down_sync(m, a.h, o), __shfl_down_sync(m, a.l, o)};
+__device__ __forceinline__ Tri32 sum_down(unsigned m, Tri32 a, int o) {
+    return {__shfl_down_sync(m, a.h, o), __shfl_down_sync(m, a.m, o), __shfl_down_sync(m, a.l, o)};
 }
 __device__ __forceinline__ double sum_down(unsigned m, double a, int o) { return __shfl_down_sync(m, a, o); }
-__device__ __forceinline__ Pair32 sum_from0(unsigned m, Pair32 a) {
-    return {__shfl_sync(m, a.h, 0), __shfl_sync(m, a.l, 0)};
+__device__ __forceinline__ Tri32 sum_from0(unsigned m, Tri32 a) {
+    return {__shfl_sync(m, a.h, 0), __shfl_sync(m, a.m, 0), __shfl_sync(m, a.l, 0)};
 }
 __device__ __forceinline__ double sum_from0(unsigned m, double a) { return __shfl_sync(m, a, 0); }
-template <typename T> struct sum_of { using type = Pair32; };
+// whole warps
+__device__ __forceinline__ Tri32 sum_xor(Tri32 a, int o) {
+    return {__shfl_xor_sync(0xffffffffu, a.h, o), __shfl_xor_sync(0xffffffffu, a.m, o), __shfl_xor_sync(0xffffffffu, a.l, o)};
+}
+__device__ __forceinline__ Tri32 sum_from(Tri32 a, int lane) {
+    return {__shfl_sync(0xffffffffu, a.h, lane), __shfl_sync(0xffffffffu, a.m, lane), __shfl_sync(0xffffffffu, a.l, lane)};
+}
+template <typename T> struct sum_of { using type = Tri32; };
 template <> struct sum_of<double> { using type = double; };
 
 // Block-wide sum of `nv` doubles per thread into out[0..nv) (thread 0 writes).
@@ -526,7 +554,7 @@ __device__ __forceinline__ void load_tw(C2* s, const C2* g, int n) {
 // copies into the other staging buffer while the current batch is computed.
 // Per line: three complex inverse transforms (u_x + i u_y, u_z + i w_x,
 // w_y + i w_z) run side by side by three thread groups; n = u x omega -
-// (chi/eta)(u - u_s) pointwise with the force/moment partial sums in double;
+// (chi/eta)(u - u_s) pointwise with the force/moment partial sums (sum_of);
 // forward transforms of (n_x + i n_y) per line and of (n_z[l] + i n_z[l+1])
 // per line pair; the result, truncated to kz < Kz, overwrites fields 0..2 of
 // B (only this batch's lines, whose input is already in shared memory).
@@ -702,11 +730,16 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
         constexpr bool SHORT = sizeof(T) == 8 ? N <= 128 : Z3 || G <= 16;
         constexpr bool EAGER = SHORT || G <= 16;
         using Sum = typename sum_of<T>::type;
-        Sum fm[6] = {};   // q and (offset from jc in cells) x q
+        // q and (offset from jc in cells) x q; FP32: the offsets along x and y from
+        // line LC of the batch, which lies in one x-plane
+        constexpr int LC = LZ > 2 ? LZ / 2 : 0;
+        static_assert(sizeof(T) == 8 || NY % LZ == 0, "a batch's lines lie in one x-plane");
+        Sum fm[6] = {};
         bool touched = false;
-        // n = u x w - (chi/eta)(u - us) of line l at z and the force sums;
+        // n = u x w - (chi/eta)(u - us) of line l + j at z and the force sums;
         // cs: chi and us there if the line is flagged
-        auto nonlinear = [&](int l, int z, int a, const T* cs, T& nx, T& ny, T& nz) {
+        auto nonlinear = [&](int l0, int j, int z, int a, const T* cs, T& nx, T& ny, T& nz) {
+            const int l = l0 + j;
             const long lid = (long)b * LZ + l;
             const C2 z0 = tile(l, 0)[a], z1 = tile(l, 1)[a], z2 = tile(l, 2)[a];
             const T ux = z0.x, uy = z0.y, uz = z1.x, wx = z1.y, wy = z2.x, wz = z2.y;
@@ -718,7 +751,6 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
                 const size_t po = (size_t)lid * N + z;
                 const T c = EAGER ? cs[0] : chi[po];
                 if (c != (T)0) {
-                    const int x = (int)(lid / nyl), y = (int)(lid % nyl);
                     const T sx = EAGER ? cs[1] : us[po], sy = EAGER ? cs[2] : us[N3 + po], sz = EAGER ? cs[3] : us[2 * N3 + po];
                     const T ce = c * inv_eta;
                     nx -= ce * (ux - sx);
@@ -726,16 +758,31 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
                     nz -= ce * (uz - sz);
                     if constexpr (!PM) {
                         const Sum qx = pen_term(c, ux, sx), qy = pen_term(c, uy, sy), qz = pen_term(c, uz, sz);
-                        const T jx = (T)(x - kp.jc[0]), jy = (T)(y - kp.jc[1]), jz = (T)(z - kp.jc[2]);
+                        const T jz = (T)(z - kp.jc[2]);
                         sum_add(fm[0], qx);
                         sum_add(fm[1], qy);
                         sum_add(fm[2], qz);
-                        sum_fma(fm[3], jy, qz);
-                        sum_fma(fm[3], -jz, qy);
-                        sum_fma(fm[4], jz, qx);
-                        sum_fma(fm[4], -jx, qz);
-                        sum_fma(fm[5], jx, qy);
-                        sum_fma(fm[5], -jy, qx);
+                        if constexpr (sizeof(T) == 8) {
+                            const int x = (int)(lid / nyl), y = (int)(lid % nyl);
+                            const T jx = (T)(x - kp.jc[0]), jy = (T)(y - kp.jc[1]);
+                            sum_fma(fm[3], jy, qz);
+                            sum_fma(fm[3], -jz, qy);
+                            sum_fma(fm[4], jz, qx);
+                            sum_fma(fm[4], -jx, qz);
+                            sum_fma(fm[5], jx, qy);
+                            sum_fma(fm[5], -jy, qx);
+                        } else {
+                            sum_fma(fm[3], -jz, qy);
+                            sum_fma(fm[4], jz, qx);
+                            if constexpr (LZ > 2) {
+                                const T jl = (T)(l - LC);
+                                sum_fma(fm[3], jl, qz);
+                                sum_fma(fm[5], -jl, qx);
+                            } else if (j == 1) {
+                                sum_add(fm[3], qz);
+                                sum_add(fm[5], neg(qx));
+                            }
+                        }
                     }
                     touched = true;
                 }
@@ -768,8 +815,8 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
                     cs[j][3] = us[2 * N3 + po];
                 }
             T nx0, ny0, nz0, nx1, ny1, nz1;
-            nonlinear(l, z, a, cs[0], nx0, ny0, nz0);
-            nonlinear(l + 1, z, a, cs[1], nx1, ny1, nz1);
+            nonlinear(l, 0, z, a, cs[0], nx0, ny0, nz0);
+            nonlinear(l, 1, z, a, cs[1], nx1, ny1, nz1);
             if constexpr (SP) {
                 // s = chi_sp omega of both lines, read before their slots are reused
                 const long lid0 = (long)b * LZ + l;
@@ -784,24 +831,13 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
             tile(l + 1, 0)[a] = cmk<C2>(nx1, ny1);
             tile(l, 1)[a] = cmk<C2>(nz0, nz1);
         }
-        // this batch's force sums: warp tree over the lanes that exist, then
-        // lane i < 6 adds sum i, compensated, to the warp's slot
+        // this batch's force sums: over the warp's lanes that exist, then one
+        // lane per sum adds it, compensated, to the warp's slot
         if (!PM && __any_sync(warp_lanes(), touched)) {
             constexpr int TAIL = 3 * LZ * G % 32;   // lanes of a last, partial warp
             static_assert(TAIL == 0 || TAIL >= 3, "two sums per lane at most");
             const unsigned m = warp_lanes();
             const int lane = threadIdx.x & 31, nl = __popc(m);
-            Sum mine[2] = {};   // the second of a lane only in a warp of fewer than six
-#pragma unroll
-            for (int i = 0; i < 6; ++i) {
-                for (int o = 16; o > 0; o >>= 1) {
-                    const Sum v = sum_down(m, fm[i], o);
-                    if (lane + o < nl) sum_add(fm[i], v);
-                }
-                const Sum v = sum_from0(m, fm[i]);
-                if (lane == i) mine[0] = v;
-                if (TAIL > 0 && TAIL < 6 && lane + nl == i) mine[1] = v;
-            }
             double* const ws = wacc[threadIdx.x >> 5];
             auto flush = [&](int i, Sum v) {
                 Acc a = {ws[2 * i], ws[2 * i + 1]};
@@ -809,8 +845,66 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
                 ws[2 * i] = a.s;
                 ws[2 * i + 1] = a.c;
             };
-            if (lane < 6) flush(lane, mine[0]);
-            if (TAIL > 0 && TAIL < 6 && lane + nl < 6) flush(lane + nl, mine[1]);
+            auto reduce = [&](int i) {   // into lane 0
+                for (int o = 16; o > 0; o >>= 1) {
+                    const Sum v = sum_down(m, fm[i], o);
+                    if (lane + o < nl) sum_add(fm[i], v);
+                }
+            };
+            bool done = false;
+            if constexpr (sizeof(T) == 4) {
+                // the offsets of line LC
+                const int x = b * LZ / nyl, y = b * LZ - x * nyl + LC;
+                const T jx = (T)(x - kp.jc[0]), jy = (T)(y - kp.jc[1]);
+                if (TAIL == 0 || nl == 32) {
+                    // a whole warp: the first exchanges halve the sums a lane keeps (8
+                    // additions of three words instead of 30; static plate at
+                    // 128^3, ten steps, 775 -> 693 us)
+                    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+                    Sum k[3];
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) {
+                        k[i] = b4 ? fm[i + 3] : fm[i];
+                        sum_add(k[i], sum_xor(b4 ? fm[i] : fm[i + 3], 16));
+                    }
+                    const Sum none = {};
+                    Sum k0 = b3 ? k[2] : k[0], k1 = b3 ? none : k[1];
+                    sum_add(k0, sum_xor(b3 ? k[0] : k[2], 8));
+                    sum_add(k1, sum_xor(b3 ? k[1] : none, 8));
+                    Sum v = b2 ? k1 : k0;
+                    sum_add(v, sum_xor(b2 ? k0 : k1, 4));
+                    sum_add(v, sum_xor(v, 2));
+                    sum_add(v, sum_xor(v, 1));
+                    // sum i is in the lanes of b4 = i / 3, (b3, b2) = (0, 0), (0, 1), (1, 0)
+                    const int i = 3 * (int)b4 + (b3 ? 2 : (int)b2);
+                    const Sum s0 = sum_from(v, 0), s1 = sum_from(v, 4), s2 = sum_from(v, 8);
+                    sum_fma(v, i == 3 ? jy : i == 4 ? -jx : i == 5 ? jx : (T)0, i == 5 ? s1 : s2);
+                    sum_fma(v, i == 5 ? -jy : (T)0, s0);
+                    if ((lane & 3) == 0 && !(b3 && b2)) flush(i, v);
+                    done = true;
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 6; ++i) reduce(i);
+                    sum_fma(fm[3], jy, fm[2]);
+                    sum_fma(fm[4], -jx, fm[2]);
+                    sum_fma(fm[5], jx, fm[1]);
+                    sum_fma(fm[5], -jy, fm[0]);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 6; ++i) reduce(i);
+            }
+            if (!done) {
+                Sum mine[2] = {};   // the second of a lane only in a warp of fewer than six
+#pragma unroll
+                for (int i = 0; i < 6; ++i) {
+                    const Sum v = sum_from0(m, fm[i]);
+                    if (lane == i) mine[0] = v;
+                    if (TAIL > 0 && TAIL < 6 && lane + nl == i) mine[1] = v;
+                }
+                if (lane < 6) flush(lane, mine[0]);
+                if (TAIL > 0 && TAIL < 6 && lane + nl < 6) flush(lane + nl, mine[1]);
+            }
         }
         __syncthreads();
         {
