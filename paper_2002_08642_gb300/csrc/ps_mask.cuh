@@ -202,9 +202,9 @@ __device__ __forceinline__ void closest_rel(const R P[3], const R b[3], const R 
     // one division for all remaining regions: an edge's or the face's parameter
     const bool e_ab = le0(vc) && ge0(d1) && le0(d3);
     const bool e_ac = !e_ab && le0(vb) && ge0(d2) && le0(d6);
-    const R l_bc = d43 + d56;   // |c - b|^2; 0: va is rounding
-    const bool e_bc = !e_ab && !e_ac && (le0(va) || le0(l_bc)) && ge0(d43) && ge0(d56);
-    const R den = e_ab ? d1 - d3 : e_ac ? d2 - d6 : e_bc ? l_bc : va + vb + vc;
+    // (d43 + d56 = |c - b|^2: with both 0, va is rounding)
+    const bool e_bc = !e_ab && !e_ac && (le0(va) || (is0(d43) && is0(d56))) && ge0(d43) && ge0(d56);
+    const R den = e_ab ? d1 - d3 : e_ac ? d2 - d6 : e_bc ? d43 + d56 : va + vb + vc;
     if (is0(den)) {
         const bool ac = cc >= bb;
         const R len = ac ? cc : bb;
@@ -260,11 +260,16 @@ __device__ __forceinline__ void tri_setup(const MaskWs& m, const MaskArgs& a, in
         }
     const double b = X[1] - X[0], c = X[2] - X[0];
     const T tb = (T)b, tc = (T)c;
-    // edge components of all three axes from the lanes of this triangle
+    // edge components of all three axes from the lanes of this triangle, and
+    // as floats (converted once per lane: a conversion is an FP64 instruction)
+    const float ob = (float)tb, oc = (float)tc;
     T vb[3], vc[3];
+    float fb[3], fc[3];
     for (int q = 0; q < 3; ++q) {
         vb[q] = __shfl_sync(all, tb, l0 + q);
         vc[q] = __shfl_sync(all, tc, l0 + q);
+        fb[q] = __shfl_sync(all, ob, l0 + q);
+        fc[q] = __shfl_sync(all, oc, l0 + q);
     }
     if (!ok || r == 3) return;
     TriGeo<T>& g = *reinterpret_cast<TriGeo<T>*>(m.geo + (size_t)t * kTriGeoBytes);
@@ -289,7 +294,7 @@ __device__ __forceinline__ void tri_setup(const MaskWs& m, const MaskArgs& a, in
     g.f[r] = f;
     g.b[r] = tb;
     g.c[r] = tc;
-    g.m[r] = ((float)b + (float)c) * (1.0f / 3.0f);
+    g.m[r] = (ob + oc) * (1.0f / 3.0f);
     if (r == 0) {
         g.bb = vb[0] * vb[0] + vb[1] * vb[1] + vb[2] * vb[2];
     } else if (r == 1) {
@@ -297,10 +302,10 @@ __device__ __forceinline__ void tri_setup(const MaskWs& m, const MaskArgs& a, in
         // sphere about the centroid
         float da = 0.0f, db = 0.0f, dc = 0.0f;
         for (int q = 0; q < 3; ++q) {
-            const float fb = (float)vb[q], fc = (float)vc[q], mq = (fb + fc) * (1.0f / 3.0f);
+            const float mq = (fb[q] + fc[q]) * (1.0f / 3.0f);
             da += mq * mq;
-            db += (fb - mq) * (fb - mq);
-            dc += (fc - mq) * (fc - mq);
+            db += (fb[q] - mq) * (fb[q] - mq);
+            dc += (fc[q] - mq) * (fc[q] - mq);
         }
         g.r = sqrtf(fmaxf(da, fmaxf(db, dc))) * 1.00001f;
     } else {
@@ -310,14 +315,13 @@ __device__ __forceinline__ void tri_setup(const MaskWs& m, const MaskArgs& a, in
                                 (float)(vb[0] * vc[1] - vb[1] * vc[0])};
             float l2 = 0.0f, bb = 0.0f, cc = 0.0f;   // squared edge lengths
             for (int q = 0; q < 3; ++q) {
-                const float fb = (float)vb[q], fc = (float)vc[q];
-                bb += fb * fb;
-                cc += fc * fc;
-                l2 += (fb - fc) * (fb - fc);
+                bb += fb[q] * fb[q];
+                cc += fc[q] * fc[q];
+                l2 += (fb[q] - fc[q]) * (fb[q] - fc[q]);
             }
             l2 = fmaxf(l2, fmaxf(bb, cc));
             const float big = fmaxf(fabsf(n[0]), fmaxf(fabsf(n[1]), fabsf(n[2])));
-            const bool plane = has_plane(big, l2, sqrtf(l2) + (float)(reach + a.dx));
+            const bool plane = has_plane(big, l2, sqrtf(l2) + (float)reach);
             const float k = plane ? 1.0f / big : 0.0f;
             const float x = n[0] * k, y = n[1] * k, z = n[2] * k, u = plane ? rsqrtf(x * x + y * y + z * z) : 0.0f;
             g.nrm[0] = x * u;
