@@ -31,7 +31,7 @@ struct LoadArgs {
 // and sin(pi(r-1/2)/2) = cos(pi(r-3/2)/2), the arguments in units of pi.
 __device__ __forceinline__ double delta_smoothed(double r) {
     r = fabs(r);
-    if (r >= 2.5) return 0.0;
+    if (!(r < 2.5)) return 0.0;   // also a node that is no number
     const bool inner = r <= 1.5;
     const double t = cospi(0.5 * (inner ? r : r - 1.5));
     return inner ? 0.25 * (1.0 + (2.0 * M_SQRT2 / M_PI) * t) : 0.25 * ((2.5 - r) - (2.0 / M_PI) * t);
