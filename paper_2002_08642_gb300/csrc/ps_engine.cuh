@@ -5,10 +5,12 @@
 #include "ps_kernels.cuh"
 #include "ps_adjoint_z.cuh"
 
-// x-inverse: at most this many (ky, kz tile) tiles take the split kernel. FP32:
-// fewer than two per SM of a GB300 (255 tiles, 128^3: plate run 705 -> 696 us;
-// 508 tiles, 192^3: pressure 237 -> 241). FP64, where the sixth transform
-// costs arithmetic: fewer than one (252 tiles, 96^3: step 489 -> 493 us)
+// x-inverse: at most this many (ky, kz tile) tiles take the split kernel. The
+// limits are cut-offs between measured sizes; no built size has a tile count
+// between them and the next one named. FP32: 255 tiles, 128^3, plate run 705 ->
+// 696 us with the split; 508 tiles, 192^3, pressure 237 -> 241. FP64, where the
+// sixth transform costs arithmetic: one tile per SM of a GB300 (64^3 62 -> 23 us
+// a pass; 252 tiles, 96^3: step 489 -> 493)
 #ifndef PS_XSPLIT_TILES
 #define PS_XSPLIT_TILES 256
 #endif
@@ -125,7 +127,7 @@ template <typename T, int N, int NZ = N> struct Engine {
         static int g = 0;
         return g;
     }
-    static int& x1grid() {
+    static int& x1grid() {   // x-inverse with the curl (k_xinv_split or k_xinv_tma)
         static int g = 0;
         return g;
     }
@@ -135,10 +137,6 @@ template <typename T, int N, int NZ = N> struct Engine {
         return g;
     }
     static int& x5agrid() {
-        static int g = 0;
-        return g;
-    }
-    static int& xsgrid() {
         static int g = 0;
         return g;
     }
@@ -152,7 +150,6 @@ template <typename T, int N, int NZ = N> struct Engine {
     }
     static constexpr size_t sm_x1 = (size_t)GE::y2_smem(GE::CX1);
     static constexpr size_t sm_x5t = (size_t)XFwd<T, N, KZ_>::smem;
-    static constexpr size_t sm_x5s = sm_x5t;   // the sponge variant keeps three result tiles
     static int& x5sgrid() {
         static int g = 0;
         return g;
@@ -166,7 +163,7 @@ template <typename T, int N, int NZ = N> struct Engine {
         const C2* tw = (const C2*)b.tw;
         if constexpr (XSPLIT) {
             const int items = kp.kyn * (KZ_ / GE::CX1) * 6;
-            launch(k_xinv_split<T, N, KZ_>, items < xsgrid() ? items : xsgrid(), thr_x1, sm_x1, s, *b.tmU, kp, (C2*)b.A, tw,
+            launch(k_xinv_split<T, N, KZ_>, items < x1grid() ? items : x1grid(), thr_x1, sm_x1, s, *b.tmU, kp, (C2*)b.A, tw,
                                                                                               b.err);
         } else {
             launch(k_xinv_tma<T, N, 6, KZ_>, x1grid(), thr_x1, sm_x1, s, *b.tmU, kp, (C2*)b.A, tw, b.err);
@@ -198,13 +195,16 @@ template <typename T, int N, int NZ = N> struct Engine {
         y2grid() = nsm * (occ < 1 ? 1 : occ);
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_yfwd_tma<T, N, GE::CY4, 3, KZ_>, thr_y4, sm_y4))) return e;
         y4grid() = nsm * (occ < 1 ? 1 : occ);
-        if ((e = attr(k_xinv_tma<T, N, 6, KZ_>, sm_x1))) return e;
         if constexpr (XSPLIT) {
             if ((e = attr(k_xinv_split<T, N, KZ_>, sm_x1))) return e;
             if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xinv_split<T, N, KZ_>, thr_x1, sm_x1)))
                 return e;
-            xsgrid() = nsm * (occ < 1 ? 1 : occ);
+        } else {
+            if ((e = attr(k_xinv_tma<T, N, 6, KZ_>, sm_x1))) return e;
+            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xinv_tma<T, N, 6, KZ_>, thr_x1, sm_x1)))
+                return e;
         }
+        x1grid() = nsm * (occ < 1 ? 1 : occ);
         if ((e = attr(k_xinv_tma<T, N, 3, KZ_>, sm_x1))) return e;
         if ((e = attr(k_xinv_tma<T, N, 1, KZ_>, sm_x1))) return e;
         if ((e = attr(k_yinv_tma<T, N, 3, KZ_>, sm_y2))) return e;
@@ -212,8 +212,8 @@ template <typename T, int N, int NZ = N> struct Engine {
         if ((e = attr(k_xfwd_tma<T, N, 0, false, KZ_>, sm_x5t))) return e;
         if ((e = attr(k_xfwd_tma<T, N, 1, false, KZ_>, sm_x5t))) return e;
         if ((e = attr(k_xfwd_tma<T, N, 2, false, KZ_>, sm_x5t))) return e;
-        if ((e = attr(k_xfwd_tma<T, N, 3, true, KZ_>, sm_x5s))) return e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xfwd_tma<T, N, 3, true, KZ_>, thr_x5, sm_x5s)))
+        if ((e = attr(k_xfwd_tma<T, N, 3, true, KZ_>, sm_x5t))) return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xfwd_tma<T, N, 3, true, KZ_>, thr_x5, sm_x5t)))
             return e;
         x5agrid() = nsm * (occ < 1 ? 1 : occ);
         if ((e = attr(k_adj_zpass<T, NZ, N>, AZ::smem))) return e;
@@ -221,14 +221,12 @@ template <typename T, int N, int NZ = N> struct Engine {
             return e;
         const int nab = N * N / 2;
         zagrid() = nsm * (occ < 1 ? 1 : occ) < nab ? nsm * (occ < 1 ? 1 : occ) : nab;
-        if ((e = attr(k_xfwd_tma<T, N, 0, true, KZ_>, sm_x5s))) return e;
+        if ((e = attr(k_xfwd_tma<T, N, 0, true, KZ_>, sm_x5t))) return e;
         if ((e = attr(k_zpass<T, NZ, false, true, N>, sm_zp))) return e;
         if ((e = attr(k_yfwd_tma<T, N, GE::CY4, 6, KZ_>, sm_y4))) return e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xfwd_tma<T, N, 0, true, KZ_>, thr_x5, sm_x5s)))
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xfwd_tma<T, N, 0, true, KZ_>, thr_x5, sm_x5t)))
             return e;
         x5sgrid() = nsm * (occ < 1 ? 1 : occ);
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xinv_tma<T, N, 6, KZ_>, thr_x1, sm_x1))) return e;
-        x1grid() = nsm * (occ < 1 ? 1 : occ);
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xinv_tma<T, N, 3, KZ_>, thr_x1, sm_x1))) return e;
         x1pgrid() = nsm * (occ < 1 ? 1 : occ);
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_xfwd_tma<T, N, 0, false, KZ_>, thr_x5, sm_x5t))) return e;
@@ -268,7 +266,7 @@ template <typename T, int N, int NZ = N> struct Engine {
         else launch(k_yfwd_tma<T, N, GE::CY4, 3, KZ_>, y4grid(), thr_y4, sm_y4, s, *b.tmB, k1, (C2*)b.A, tw, b.err);
         if (ev) { cudaEventRecord(ev[7], s); cudaEventRecord(ev[8], s); }
         if (sp)
-            launch(k_xfwd_tma<T, N, 0, true, KZ_>, x5sgrid(), thr_x5, sm_x5s, s, *b.tmA5, *b.tmUp, *b.tmHp, kp, (C2*)b.U,
+            launch(k_xfwd_tma<T, N, 0, true, KZ_>, x5sgrid(), thr_x5, sm_x5t, s, *b.tmA5, *b.tmUp, *b.tmHp, kp, (C2*)b.U,
                                                                        (C2*)b.H, (const T*)b.Ex, (const T*)b.Ez,
                                                                        first, tw, b.err);
         else
@@ -317,7 +315,7 @@ template <typename T, int N, int NZ = N> struct Engine {
                                                                      (const T*)b.us, b.flag, (T*)gchi, (T*)gus,
                                                                      twz(b.tw), b.err);
         launch(k_yfwd_tma<T, N, GE::CY4, 6, KZ_>, y4grid(), thr_y4, sm_y4, s, *b.tmB, k1, (C2*)b.A, tw, b.err);
-        launch(k_xfwd_tma<T, N, 3, true, KZ_>, x5agrid(), thr_x5, sm_x5s, s, *b.tmA5, *b.tmL, *b.tmL, k1, (C2*)lam, (C2*)mu,
+        launch(k_xfwd_tma<T, N, 3, true, KZ_>, x5agrid(), thr_x5, sm_x5t, s, *b.tmA5, *b.tmL, *b.tmL, k1, (C2*)lam, (C2*)mu,
                                                                        (const T*)b.Ex, (const T*)b.Ez, aw.first, tw,
                                                                        b.err);
         return cudaGetLastError();

@@ -160,8 +160,7 @@ __host__ __device__ constexpr int pow2_part(int n) {
     return p;
 }
 // Largest radix of a line's power-of-two stages. Long lines: 16 (fewest
-// shared-memory round trips). Short lines (n <= 64 and the n = 3M lines over
-// them): 4, so that a line has n / 4 threads instead of n / 16. Radix 4 costs
+// shared-memory round trips). Short lines (n <= 64, FP64 n <= 96): 4, so that a line has n / 4 threads instead of n / 16. Radix 4 costs
 // about the same arithmetic per point there (FP64, n = 32: 15 operations
 // against 14), and the passes of small grids are one chain of a few warps per
 // SM.

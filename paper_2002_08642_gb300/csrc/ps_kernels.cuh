@@ -725,8 +725,11 @@ k_zpass(KP kp, cplx<T>* __restrict__ B, const T* __restrict__ chi, const T* __re
         __syncthreads();
         // one buffer: every read of it is done, the next batch may land
         if (!Z3 && NB == 1 && threadIdx.x == 0 && more) issue(b + gridDim.x, 0);
-        // lines whose pass gains from the flagged lines' loads ahead of their
-        // use and from forward transforms in the first groups: see there
+        // lines whose pass gains from forward transforms in the first groups
+        // (SHORT) and from the flagged lines' loads ahead of their use (EAGER).
+        // Measured limits, each with its two sides where it is used below; why
+        // lines of 384 and 768 points gain where 512 loses was not found (all
+        // three run at two or three blocks per SM and 72 to 80 registers)
         constexpr bool SHORT = sizeof(T) == 8 ? N <= 128 : Z3 || G <= 16;
         constexpr bool EAGER = SHORT || G <= 16;
         using Sum = typename sum_of<T>::type;
