@@ -43,8 +43,10 @@ template <typename T, int N> struct AdjZ {
 // Memory: fifteen z-spectral fields and eight physical ones cross HBM once;
 // as separate inverse transforms, pointwise kernel and forward transforms
 // thirty more physical fields went out and came back (GB300, 512^3 FP32: three
-// inverse, one pointwise and two forward kernels 4.29 ms, this 2.96 ms; it is
-// bound by its fifteen line transforms' shared memory and barriers).
+// inverse, one pointwise and two forward kernels 4.29 ms, this 2.96 ms). It is
+// bound by its fifteen line transforms' exchanges through shared memory: at 384 x
+// 384 x 192 184 M wavefronts in 0.71 ms, 83 % of the SMs' rate, 37 % of them bank
+// conflicts; issue slots 54 %, DRAM 34 %.
 template <typename T, int N, int NY = N>
 __global__ void __launch_bounds__(AdjZ<T, N>::threads, AdjZ<T, N>::minb)
 k_adj_zpass(KP kp, AdjW aw, cplx<T>* __restrict__ B, const cplx<T>* __restrict__ NB, const T* __restrict__ chi,
