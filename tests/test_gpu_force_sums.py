@@ -10,9 +10,8 @@ sum of FP32 words of 48 bits is off by up to 2^-49 of a single term's moment, a
 plain FP32 sum by 2^-25 or more. With u_s of both signs the terms cancel; the
 moment point lies in the body or far outside the box.
 
-Velocities that are not zero cannot be isolated that way (the z pass has its
-own rounding of u); u_s then is chosen close to -u's size, and FP32 force is
-compared with FP64 in the step tests.
+With a flow the z pass rounds u itself; the last test compares an FP32 with an
+FP64 context where the terms cancel.
 """
 from fractions import Fraction
 
